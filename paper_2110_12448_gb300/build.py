@@ -16,7 +16,10 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libpf.so")
 OUT_DIR_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(OUT_DIR_CHECKED, "libpf.so")
-SOURCES = ["step2d.cu", "step3d.cu", "observe.cu", "pf_api.cu"]
+# (source, object, extra flags): the 2D step kernels once per precision and scheme
+SOURCES = [("step2d_inst.cu", f"step2d_{t}_{s.lower()}.o", [f"-DPF_REAL={t}", f"-DPF_SCHEME={s}"])
+           for t in ("double", "float") for s in ("S21", "SBAR21", "S10")]
+SOURCES += [(s, s.replace(".cu", ".o"), []) for s in ("step2d.cu", "step2d_c.cu", "step3d.cu", "observe.cu", "pf_api.cu")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 
@@ -44,15 +47,15 @@ def build(force: bool = False, verbose: bool = False, extra_flags=(), checked: b
     headers.append(os.path.join(os.path.dirname(HERE), "include", "pf.h"))
     objs = []
     jobs = []
-    for src in SOURCES:
+    for src, obj, defs in SOURCES:
         s = os.path.join(CSRC, src)
-        o = os.path.join(out_dir, src.replace(".cu", ".o"))
+        o = os.path.join(out_dir, obj)
         objs.append(o)
         if force or not _newer(o, [s] + headers):
-            cmd = [nvcc(), *ARCH, *FLAGS, *extra_flags, "-c", s, "-o", o]
+            cmd = [nvcc(), *ARCH, *FLAGS, *extra_flags, *defs, "-c", s, "-o", o]
             jobs.append(cmd)
     if jobs:
-        with cf.ThreadPoolExecutor(max_workers=len(jobs)) as ex:
+        with cf.ThreadPoolExecutor(max_workers=min(len(jobs), os.cpu_count() or 4)) as ex:
             futs = [ex.submit(subprocess.run, c, capture_output=True, text=True) for c in jobs]
             for c, f in zip(jobs, futs):
                 r = f.result()

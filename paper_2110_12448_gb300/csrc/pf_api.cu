@@ -172,6 +172,7 @@ struct pf_sim {
     void* rate;  // d psi/dt of the two-kernel form (nullptr when fused)
     int n_grains;
     int gmax;         // largest grain index in the map (0: every cell in grain 0)
+    bool orthonormal; // every grain's upper 2x2 block is (2D)
     int64_t rec_gen;  // advanced by every change the instance record carries
     std::vector<double> rot_h, centres_h;
     int64_t step;
@@ -212,24 +213,37 @@ void build_work(const pf_sim* s, int inst, std::vector<WorkItem>& out) {
     }
 }
 
-// the 2D kernel variant: 1 frozen temperature and/or periodic x (either time
-// level), 2 isothermal with mirror walls at the T0 level, 0 otherwise
-int ds_of(const pf_params& p) {
-    if (p.thermal == PF_FROZEN_GRADIENT || p.bc_x == PF_BC_PERIODIC) return 1;
-    return p.time_level == PF_T0 ? 2 : 0;
+// The 2D kernel of an instance.  Variant: 1 frozen temperature and/or periodic
+// x (either time level), 2 isothermal with mirror walls at the T0 level, 0
+// otherwise.  Frames: 0 every cell in grain 0 and its matrix orthonormal, 1
+// grain maps with orthonormal matrices, 2 any matrices (compiled for variant 1,
+// which takes isothermal instances and both time levels too).
+struct Path {
+    int var, fr;
+};
+Path path_of(const pf_sim* s) {
+    Path k{0, 0};
+    if (s->p.dim == 3) return k;
+    if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.bc_x == PF_BC_PERIODIC) k.var = 1;
+    else k.var = s->p.time_level == PF_T0 ? 2 : 0;
+    if (s->p.precision == PF_F32C) return k;  // its kernel takes any frames
+    k.fr = s->gmax == 0 ? 0 : 1;
+    if (!s->orthonormal) k = Path{1, 2};
+    return k;
 }
 
 // resident units of the step's kernel; for the two-kernel form those of the
 // pass with fewer, so that one persistent grid serves both passes
-int occupancy_of(const pf_params& p, int bx, int by) {
-    const int prec = kprec(p);
-    if (p.dim == 3) return occupancy_step3d(prec, p.scheme, bx, by);
-    if (p.kernels == PF_TWO_KERNELS)
-        return std::min(occupancy_step2d(prec, p.scheme, bx, ds_of(p), 1), occupancy_step2d(prec, p.scheme, bx, ds_of(p), 2));
-    return occupancy_step2d(prec, p.scheme, bx, ds_of(p));
+int occupancy_of(int dim, int prec, int scheme, int bx, int by, const Path& k, bool two) {
+    if (dim == 3) return occupancy_step3d(prec, scheme, bx, by);
+    if (two)
+        return std::min(occupancy_step2d(prec, scheme, bx, k.var, k.fr, 1), occupancy_step2d(prec, scheme, bx, k.var, k.fr, 2));
+    return occupancy_step2d(prec, scheme, bx, k.var, k.fr);
 }
 
-int occupancy(const pf_sim* s) { return occupancy_of(s->p, s->bx, s->by); }
+int occupancy(const pf_sim* s) {
+    return occupancy_of(s->p.dim, kprec(s->p), s->p.scheme, s->bx, s->by, path_of(s), s->p.kernels == PF_TWO_KERNELS);
+}
 
 InstRec make_rec(const pf_sim* s, int parity_offset) {
     InstRec r{};
@@ -278,6 +292,18 @@ InstRec make_rec(const pf_sim* s, int parity_offset) {
     c[C_D] = s->p.D;
     c[C_ISQ2DT] = 1.0 / (1.41421356237309504880 * s->p.dt);
     c[C_I4H2] = 1.0 / (4.0 * h * h);
+    c[C_OPK] = 1.0 + s->p.k;
+    const double sq2 = 1.41421356237309504880;
+    c[C_DTL21] = s->p.dt / (6.0 * h * h);
+    c[C_DTL10] = s->p.dt / (h * h);
+    c[C_SQ21] = sq2 * 6.0 * h * h;
+    c[C_SQ10] = sq2 * h * h;
+    c[C_LAM21] = sq2 * s->p.lambda * 6.0 * h * h;
+    c[C_LAM10] = sq2 * s->p.lambda * h * h;
+    c[C_UD21] = s->p.dt * s->p.D / (24.0 * h * h);
+    c[C_UD10] = s->p.dt * s->p.D / (h * h);
+    c[C_UA21] = 1.0 / (24.0 * sq2 * h * h);
+    c[C_UA10] = 4.0 / (sq2 * h);
     for (int i = 0; i < NC; ++i) {
         r.cd[i] = c[i];
         r.cf[i] = (float)c[i];
@@ -303,11 +329,28 @@ int upload_work(pf_sim* s) {
 
 int upload_rot(pf_sim* s) {
     const int n = s->n_grains;
+    std::vector<double> r(s->rot_h);
+    s->orthonormal = true;
+    if (s->p.dim == 2) {
+        // The 2D kernels evaluate J - g from the reflection about the crystal
+        // axes, (C2, S2) in the matrix's unused slots 6 and 7, which is exact for
+        // orthonormal frames; a frame further off than the field precision's
+        // rounding takes the kernel for any matrices.
+        const double tol = s->p.precision == PF_F64 ? 1e-14 : 2e-7;
+        for (int g = 0; g < n; ++g) {
+            double* R = &r[9 * g];
+            if (!(std::fabs(R[0] * R[0] + R[1] * R[1] - 1.0) <= tol && std::fabs(R[3] * R[3] + R[4] * R[4] - 1.0) <= tol &&
+                  std::fabs(R[0] * R[3] + R[1] * R[4]) <= tol))
+                s->orthonormal = false;
+            R[6] = R[0] * R[0] - R[1] * R[1];
+            R[7] = R[0] * R[3] - R[1] * R[4];
+        }
+    }
     if (s->p.precision == PF_F64) {
-        CK(cudaMemcpyAsync(s->rot, s->rot_h.data(), (size_t)n * 9 * sizeof(double), cudaMemcpyHostToDevice, s->st));
+        CK(cudaMemcpyAsync(s->rot, r.data(), (size_t)n * 9 * sizeof(double), cudaMemcpyHostToDevice, s->st));
         CK(cudaStreamSynchronize(s->st));
     } else {
-        std::vector<float> f(s->rot_h.begin(), s->rot_h.end());
+        std::vector<float> f(r.begin(), r.end());
         CK(cudaMemcpyAsync(s->rot, f.data(), (size_t)n * 9 * sizeof(float), cudaMemcpyHostToDevice, s->st));
         CK(cudaStreamSynchronize(s->st));
     }
@@ -319,14 +362,13 @@ bool launch_sim_step(const pf_sim* s, int64_t step) {
     const int prec = kprec(s->p);
     const int lp = (int)(step & 1);
     const StepClock clk{nullptr, nullptr, (long long)step};
+    const Path k = path_of(s);
     if (s->p.dim == 2 && s->p.kernels == PF_TWO_KERNELS)
-        return launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk,
-                             ds_of(s->p), 1) &&
-               launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk,
-                             ds_of(s->p), 2);
+        return launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk, k.var, k.fr,
+                             1) &&
+               launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk, k.var, k.fr, 2);
     if (s->p.dim == 2)
-        return launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk,
-                             ds_of(s->p));
+        return launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk, k.var, k.fr);
     return launch_step3d(prec, s->p.scheme, s->bx, s->by, s->grid, s->st, s->work, s->n_work, s->rec, lp,
                          StepClock{nullptr, nullptr, (long long)step});
 }
@@ -398,6 +440,7 @@ int pf_create(const pf_params* p, void* dev_mem, size_t bytes, void* stream, pf_
     s->rate = p->kernels == PF_TWO_KERNELS ? s->base + L.rate : nullptr;
     s->n_grains = 1;
     s->gmax = 0;  // the grain map starts zero-filled
+    s->orthonormal = true;
     s->rec_gen = 0;
     s->rot_h.assign(9, 0.0);
     s->rot_h[0] = s->rot_h[4] = s->rot_h[8] = 1.0;
@@ -846,15 +889,20 @@ int pf_get_tile(pf_sim* s, int* block_x, int* block_y, int* sweep) {
 
 int pf_debug_bounds(unsigned long long* failures, int* first_line) {
     if (!failures || !first_line) return PF_ERR_INVALID;
-    unsigned long long c[3] = {0, 0, 0};
-    int l[3] = {0, 0, 0};
-    const int r0 = bounds_step2d(&c[0], &l[0]);
-    const int r1 = bounds_step3d(&c[1], &l[1]);
-    const int r2 = bounds_observe(&c[2], &l[2]);
-    if (r0 < 0 || r1 < 0 || r2 < 0) return PF_ERR_CUDA;
-    *failures = c[0] + c[1] + c[2];
-    *first_line = l[0] ? l[0] : (l[1] ? l[1] : l[2]);
-    return (r0 == 1 && r1 == 1 && r2 == 1) ? PF_ERR_STATE : PF_OK;
+    unsigned long long c[4] = {0, 0, 0, 0};
+    int l[4] = {0, 0, 0, 0};
+    const int r[4] = {bounds_step2d(&c[0], &l[0]), bounds_step2c(&c[1], &l[1]), bounds_step3d(&c[2], &l[2]),
+                      bounds_observe(&c[3], &l[3])};
+    *failures = 0;
+    *first_line = 0;
+    bool checked = false;
+    for (int i = 0; i < 4; ++i) {
+        if (r[i] < 0) return PF_ERR_CUDA;
+        checked |= r[i] != 1;
+        *failures += c[i];
+        if (*first_line == 0) *first_line = l[i];
+    }
+    return checked ? PF_OK : PF_ERR_STATE;
 }
 
 int pf_debug_inject_launch_failure(long long after_steps) {
@@ -982,7 +1030,7 @@ struct pf_group {
     bool dirty;
     struct Cls {
         int dim, scheme, prec, bx, by, w0, n, grid;
-        int ds;    // 2D kernel variant (ds_of: 0 isothermal T1, 1 frozen temperature / periodic x, 2 isothermal T0)
+        Path path; // 2D kernel: variant and frames (the most general of the members')
         bool two;  // two-kernel form: the psi pass, then the U pass
         int occ;   // resident units per SM
         std::vector<int> boff;  // depth 2: work items of band b are [w0 + boff[b], w0 + boff[b + 1])
@@ -1018,7 +1066,7 @@ int group_rebuild(pf_group* g) {
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     auto key = [&](int i) {
         const pf_sim* s = g->members[i];
-        return ((long long)s->p.kernels << 52) | ((long long)ds_of(s->p) << 48) | ((long long)s->p.dim << 40) |
+        return ((long long)s->p.kernels << 52) | ((long long)path_of(s).var << 48) | ((long long)s->p.dim << 40) |
                ((long long)s->p.scheme << 32) |
                ((long long)s->p.precision << 24) | ((long long)s->bx << 12) | (long long)s->by;
     };
@@ -1044,10 +1092,11 @@ int group_rebuild(pf_group* g) {
         const long long k = key(i);
         if (k != prev) {
             pf_group::Cls c{s->p.dim, s->p.scheme, kprec(s->p), s->bx, s->by, (int)work.size(), 0, 0,
-                            ds_of(s->p), s->p.kernels == PF_TWO_KERNELS, 0, {}};
+                            path_of(s), s->p.kernels == PF_TWO_KERNELS, 0, {}};
             g->classes.push_back(c);
             prev = k;
         }
+        g->classes.back().path.fr = std::max(g->classes.back().path.fr, path_of(s).fr);
         const size_t first = work.size();
         build_work(s, i, work);
         g->classes.back().n = (int)work.size() - g->classes.back().w0;
@@ -1074,10 +1123,7 @@ int group_rebuild(pf_group* g) {
         }
     }
     for (auto& c : g->classes) {
-        int occ = c.dim == 3 ? occupancy_step3d(c.prec, c.scheme, c.bx, c.by)
-                  : c.two    ? std::min(occupancy_step2d(c.prec, c.scheme, c.bx, c.ds, 1),
-                                        occupancy_step2d(c.prec, c.scheme, c.bx, c.ds, 2))
-                             : occupancy_step2d(c.prec, c.scheme, c.bx, c.ds);
+        const int occ = occupancy_of(c.dim, c.prec, c.scheme, c.bx, c.by, c.path, c.two);
         if (occ <= 0) return PF_ERR_INVALID;
         c.occ = occ;
         c.grid = std::min(c.n, occ * num_sms());
@@ -1110,12 +1156,12 @@ bool group_launch_once(pf_group* g, int launch_parity) {
                                clk);
         else if (c.two)
             ok = launch_step2d(c.prec, c.scheme, c.bx, c.grid, g->st, g->work + c.w0, c.n, g->recs, launch_parity, clk,
-                               c.ds, 1) &&
+                               c.path.var, c.path.fr, 1) &&
                  launch_step2d(c.prec, c.scheme, c.bx, c.grid, g->st, g->work + c.w0, c.n, g->recs, launch_parity, clk,
-                               c.ds, 2);
+                               c.path.var, c.path.fr, 2);
         else
             ok = launch_step2d(c.prec, c.scheme, c.bx, c.grid, g->st, g->work + c.w0, c.n, g->recs, launch_parity, clk,
-                               c.ds);
+                               c.path.var, c.path.fr);
         if (!ok) return false;
     }
     if (g->thermal_any && launch_tick(g->clock, g->st) != cudaSuccess) return false;
@@ -1133,7 +1179,7 @@ bool group_launch_band(pf_group* g, int launch_parity, int b) {
         const bool ok = c.dim == 3 ? launch_step3d(c.prec, c.scheme, c.bx, c.by, grid, g->st, g->work + c.w0 + lo, cnt,
                                                    g->recs, launch_parity, clk)
                                    : launch_step2d(c.prec, c.scheme, c.bx, grid, g->st, g->work + c.w0 + lo, cnt,
-                                                   g->recs, launch_parity, clk, c.ds);
+                                                   g->recs, launch_parity, clk, c.path.var, c.path.fr);
         if (!ok) return false;
     }
     return true;

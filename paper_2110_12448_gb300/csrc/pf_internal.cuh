@@ -28,6 +28,17 @@ enum : int {
     C_D,         // D
     C_ISQ2DT,    // 1/(sqrt2 dt)
     C_I4H2,      // 1/(4h^2)
+    C_OPK,       // 1+k
+    C_DTL21,     // dt / (6h^2): Eq. PF_a in units of 1/(6h^2)
+    C_DTL10,     // dt / h^2
+    C_SQ21,      // sqrt2 6h^2
+    C_SQ10,      // sqrt2 h^2
+    C_LAM21,     // sqrt2 lambda 6h^2
+    C_LAM10,     // sqrt2 lambda h^2
+    C_UD21,      // dt D / (24 h^2): the D~_{2,1} sum's factor in the U update
+    C_UD10,      // dt D / h^2
+    C_UA21,      // 1 / (24 sqrt2 h^2): the anti-trapping sums', with alpha's 1/(sqrt2 dt)
+    C_UA10,      // 1 / (sqrt2 h): likewise, the <10> form normalised by |grad psi| h
     NC
 };
 
@@ -99,6 +110,7 @@ __device__ __forceinline__ long long pf_chk(long long i, long long n, int line) 
 #endif
 // host readers of the per-unit records (return 1 in an unchecked build)
 int bounds_step2d(unsigned long long* count, int* line);
+int bounds_step2c(unsigned long long* count, int* line);
 int bounds_step3d(unsigned long long* count, int* line);
 int bounds_observe(unsigned long long* count, int* line);
 
@@ -128,15 +140,18 @@ struct StepClock {
 // temperature and/or periodic x (T1 or T0 read from the record); 2 isothermal,
 // mirror walls, T0.  mode: 0 the fused step; 1, 2 the psi and U passes of the
 // two-kernel form (T0 time level: variant 1 or 2, prec 0 or 1)
+// fr: the crystal frames the 2D kernel is compiled for: 0 every cell of every
+// instance in grain 0 with an orthonormal frame, 1 grain maps with orthonormal
+// frames, 2 any matrices (variant 1 only; precision 2 takes any and ignores it)
 bool launch_step2d(int prec, int scheme, int bx, int grid, cudaStream_t st, const WorkItem* work, int n_work,
-                   const InstRec* recs, int launch_parity, StepClock clk, int var, int mode = 0);
+                   const InstRec* recs, int launch_parity, StepClock clk, int var, int fr, int mode = 0);
 bool launch_step3d(int prec, int scheme, int bx, int by, int grid, cudaStream_t st, const WorkItem* work,
                    int n_work, const InstRec* recs, int launch_parity, StepClock clk);
 // clock += 1 (one thread)
 cudaError_t launch_tick(long long* clock, cudaStream_t st);
 // Blocks of the fused kernel that fit on one SM (0 if not compiled); var as
 // for launch_step2d
-int occupancy_step2d(int prec, int scheme, int bx, int var, int mode = 0);
+int occupancy_step2d(int prec, int scheme, int bx, int var, int fr, int mode = 0);
 int occupancy_step3d(int prec, int scheme, int bx, int by);
 
 // Observation / initialisation kernels (observe.cu).
