@@ -75,7 +75,7 @@ template <> struct M<float> {
     // tanh(x / sqrt2) = 1 - 2 / (1 + e^{sqrt2 x}) = 1 - 2 / (1 + 2^{sqrt2 log2(e) x});
     // absolute error ~2e-7 over the whole range
     static __device__ __forceinline__ float tanh_isq2(float x) {
-        const float e = ex2_approx(x * 2.0402467570003297f);  // sqrt2 * log2(e)
+        const float e = ex2_approx(x * 2.0402788931935790f);  // sqrt2 * log2(e)
         return fmaf(-2.0f, rcp_approx(1.0f + e), 1.0f);
     }
     static __device__ __forceinline__ float rcp(float x) { return rcp_approx(x); }
