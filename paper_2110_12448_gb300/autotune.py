@@ -40,7 +40,8 @@ def work_items(w, tile) -> int:
     library's decomposition: 2D (block_x - 4)-column strips times sweep-row
     bands; 3D (block_x - 4) x (block_y - 4) columns times sweep-plane bands."""
     bx, by, sw = tile
-    n = -(-w.nx // (bx - 4)) * -(-(w.ny if w.dim == 2 else w.nz) // sw)
+    cols = w.nx if w.dim == 2 else w.nx + 1  # a 3D strip's outputs start one column before its origin
+    n = -(-cols // (bx - 4)) * -(-(w.ny if w.dim == 2 else w.nz) // sw)
     return n if w.dim == 2 else n * -(-w.ny // (by - 4))
 
 

@@ -113,6 +113,12 @@ int max_work_items(const pf_params* p) {
     return cdiv(p->nx, 12) * cdiv(p->ny, 4) * cdiv(p->nz, 4);
 }
 
+// whether d psi/dt travels between the passes in device memory: the 2D two-kernel
+// form, and 3D at the T0 level (whose delta phi takes it before psi' is rounded)
+bool stores_rate(const pf_params* p) {
+    return p->kernels == PF_TWO_KERNELS || (p->dim == 3 && p->time_level == PF_T0);
+}
+
 Layout layout(const pf_params* p) {
     Layout L{};
     L.N = (size_t)cells(p);
@@ -137,7 +143,7 @@ Layout layout(const pf_params* p) {
     L.result = take(sizeof(ObsPartial));
     L.work = take((size_t)L.max_work * sizeof(WorkItem));
     L.rec = take(sizeof(InstRec));
-    L.rate = p->kernels == PF_TWO_KERNELS ? take(L.N * L.esz) : 0;  // d psi/dt between the two kernels
+    L.rate = stores_rate(p) ? take(L.N * L.esz) : 0;  // d psi/dt between the two passes
     L.total = o;
     return L;
 }
@@ -176,7 +182,7 @@ struct pf_sim {
     int64_t rec_gen;  // advanced by every change the instance record carries
     std::vector<double> rot_h, centres_h;
     int64_t step;
-    int bx, by, sweep, n_work, grid;
+    int bx, by, sweep, n_work, grid, grid_u;  // grid_u: the 3D U pass
     bool work_dirty;
     std::vector<WorkItem> work_h;
     std::vector<int> have_prev;       // per grain + 2 (index 0: pulling axis, 1: global)
@@ -206,10 +212,11 @@ void build_work(const pf_sim* s, int inst, std::vector<WorkItem>& out) {
         for (int y0 = 0; y0 < p.ny; y0 += s->sweep)
             for (int x0 = 0; x0 < p.nx; x0 += TX) out.push_back(WorkItem{inst, x0, y0, 0, s->sweep, 0, 0, 0});
     } else {
+        // a strip's outputs are the columns x0 - 1 .. x0 + TX - 2
         const int TX = s->bx - 4, TY = s->by - 4;
         for (int z0 = 0; z0 < p.nz; z0 += s->sweep)
             for (int y0 = 0; y0 < p.ny; y0 += TY)
-                for (int x0 = 0; x0 < p.nx; x0 += TX) out.push_back(WorkItem{inst, x0, y0, z0, s->sweep, 0, 0, 0});
+                for (int x0 = 0; x0 < p.nx + 1; x0 += TX) out.push_back(WorkItem{inst, x0, y0, z0, s->sweep, 0, 0, 0});
     }
 }
 
@@ -217,32 +224,37 @@ void build_work(const pf_sim* s, int inst, std::vector<WorkItem>& out) {
 // x (either time level), 2 isothermal with mirror walls at the T0 level, 0
 // otherwise.  Frames: 0 every cell in grain 0 and its matrix orthonormal, 1
 // grain maps with orthonormal matrices, 2 any matrices (compiled for variant 1,
-// which takes isothermal instances and both time levels too).
+// which takes isothermal instances and both time levels too).  3D: frames 0 or 1.
 struct Path {
     int var, fr;
 };
 Path path_of(const pf_sim* s) {
-    Path k{0, 0};
-    if (s->p.dim == 3) return k;
+    Path k{0, s->gmax == 0 ? 0 : 1};
+    if (s->p.dim == 3) return k;  // any matrices
     if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.bc_x == PF_BC_PERIODIC) k.var = 1;
     else k.var = s->p.time_level == PF_T0 ? 2 : 0;
     if (s->p.precision == PF_F32C) return k;  // its kernel takes any frames
-    k.fr = s->gmax == 0 ? 0 : 1;
     if (!s->orthonormal) k = Path{1, 2};
     return k;
 }
 
-// resident units of the step's kernel; for the two-kernel form those of the
-// pass with fewer, so that one persistent grid serves both passes
-int occupancy_of(int dim, int prec, int scheme, int bx, int by, const Path& k, bool two) {
-    if (dim == 3) return occupancy_step3d(prec, scheme, bx, by);
+// resident units of the step's kernel; for the 2D two-kernel form those of the
+// pass with fewer, so that one persistent grid serves both passes; in 3D those
+// of the psi pass (u_pass: of the U pass)
+int occupancy_of(int dim, int prec, int scheme, int bx, int by, const Path& k, bool two, int* u_pass = nullptr) {
+    if (dim == 3) {
+        int psi = 0, u = 0;
+        const bool ok = occupancy_step3d(prec, scheme, bx, by, k.fr, psi, u);
+        if (u_pass) *u_pass = u;
+        return ok ? psi : 0;
+    }
     if (two)
         return std::min(occupancy_step2d(prec, scheme, bx, k.var, k.fr, 1), occupancy_step2d(prec, scheme, bx, k.var, k.fr, 2));
     return occupancy_step2d(prec, scheme, bx, k.var, k.fr);
 }
 
-int occupancy(const pf_sim* s) {
-    return occupancy_of(s->p.dim, kprec(s->p), s->p.scheme, s->bx, s->by, path_of(s), s->p.kernels == PF_TWO_KERNELS);
+int occupancy(const pf_sim* s, int* u_pass = nullptr) {
+    return occupancy_of(s->p.dim, kprec(s->p), s->p.scheme, s->bx, s->by, path_of(s), s->p.kernels == PF_TWO_KERNELS, u_pass);
 }
 
 InstRec make_rec(const pf_sim* s, int parity_offset) {
@@ -304,6 +316,10 @@ InstRec make_rec(const pf_sim* s, int parity_offset) {
     c[C_UD10] = s->p.dt * s->p.D / (h * h);
     c[C_UA21] = 1.0 / (24.0 * sq2 * h * h);
     c[C_UA10] = 4.0 / (sq2 * h);
+    c[C_UD120] = s->p.dt * s->p.D / (192.0 * h * h);
+    c[C_UD100] = s->p.dt * s->p.D / (2.0 * h * h);
+    c[C_UA120] = 1.0 / (192.0 * sq2 * h * h);
+    c[C_UA100] = 2.0 / (sq2 * h);
     for (int i = 0; i < NC; ++i) {
         r.cd[i] = c[i];
         r.cf[i] = (float)c[i];
@@ -320,9 +336,11 @@ int upload_work(pf_sim* s) {
     InstRec r = make_rec(s, 0);
     CK(cudaMemcpyAsync(s->rec, &r, sizeof(r), cudaMemcpyHostToDevice, s->st));
     CK(cudaStreamSynchronize(s->st));
-    const int occ = occupancy(s);
+    int occ_u = 0;
+    const int occ = occupancy(s, &occ_u);
     if (occ <= 0) return PF_ERR_INVALID;
     s->grid = std::min(s->n_work, occ * num_sms());
+    s->grid_u = std::min(s->n_work, occ_u * num_sms());
     s->work_dirty = false;
     return PF_OK;
 }
@@ -369,8 +387,8 @@ bool launch_sim_step(const pf_sim* s, int64_t step) {
                launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk, k.var, k.fr, 2);
     if (s->p.dim == 2)
         return launch_step2d(prec, s->p.scheme, s->bx, s->grid, s->st, s->work, s->n_work, s->rec, lp, clk, k.var, k.fr);
-    return launch_step3d(prec, s->p.scheme, s->bx, s->by, s->grid, s->st, s->work, s->n_work, s->rec, lp,
-                         StepClock{nullptr, nullptr, (long long)step});
+    return launch_step3d(prec, s->p.scheme, s->bx, s->by, s->st,
+                         Step3DArgs{s->work, s->n_work, s->rec, lp, clk, k.fr, s->grid, s->grid_u});
 }
 
 // Compensated FP32 state (PF_F32C): the 8 bytes per cell of a level hold the
@@ -437,7 +455,7 @@ int pf_create(const pf_params* p, void* dev_mem, size_t bytes, void* stream, pf_
     s->result = reinterpret_cast<ObsPartial*>(s->base + L.result);
     s->work = reinterpret_cast<WorkItem*>(s->base + L.work);
     s->rec = reinterpret_cast<InstRec*>(s->base + L.rec);
-    s->rate = p->kernels == PF_TWO_KERNELS ? s->base + L.rate : nullptr;
+    s->rate = stores_rate(p) ? s->base + L.rate : nullptr;
     s->n_grains = 1;
     s->gmax = 0;  // the grain map starts zero-filled
     s->orthonormal = true;
@@ -1032,7 +1050,7 @@ struct pf_group {
         int dim, scheme, prec, bx, by, w0, n, grid;
         Path path; // 2D kernel: variant and frames (the most general of the members')
         bool two;  // two-kernel form: the psi pass, then the U pass
-        int occ;   // resident units per SM
+        int occ, occ_u;  // resident units per SM (occ_u: the 3D U pass)
         std::vector<int> boff;  // depth 2: work items of band b are [w0 + boff[b], w0 + boff[b + 1])
     };
     std::vector<Cls> classes;
@@ -1092,7 +1110,7 @@ int group_rebuild(pf_group* g) {
         const long long k = key(i);
         if (k != prev) {
             pf_group::Cls c{s->p.dim, s->p.scheme, kprec(s->p), s->bx, s->by, (int)work.size(), 0, 0,
-                            path_of(s), s->p.kernels == PF_TWO_KERNELS, 0, {}};
+                            path_of(s), s->p.kernels == PF_TWO_KERNELS, 0, 0, {}};
             g->classes.push_back(c);
             prev = k;
         }
@@ -1123,7 +1141,7 @@ int group_rebuild(pf_group* g) {
         }
     }
     for (auto& c : g->classes) {
-        const int occ = occupancy_of(c.dim, c.prec, c.scheme, c.bx, c.by, c.path, c.two);
+        const int occ = occupancy_of(c.dim, c.prec, c.scheme, c.bx, c.by, c.path, c.two, &c.occ_u);
         if (occ <= 0) return PF_ERR_INVALID;
         c.occ = occ;
         c.grid = std::min(c.n, occ * num_sms());
@@ -1152,8 +1170,9 @@ bool group_launch_once(pf_group* g, int launch_parity) {
         if (c.n == 0) continue;
         bool ok;
         if (c.dim == 3)
-            ok = launch_step3d(c.prec, c.scheme, c.bx, c.by, c.grid, g->st, g->work + c.w0, c.n, g->recs, launch_parity,
-                               clk);
+            ok = launch_step3d(c.prec, c.scheme, c.bx, c.by, g->st,
+                               Step3DArgs{g->work + c.w0, c.n, g->recs, launch_parity, clk, c.path.fr, c.grid,
+                                          std::min(c.n, c.occ_u * num_sms())});
         else if (c.two)
             ok = launch_step2d(c.prec, c.scheme, c.bx, c.grid, g->st, g->work + c.w0, c.n, g->recs, launch_parity, clk,
                                c.path.var, c.path.fr, 1) &&
@@ -1168,31 +1187,48 @@ bool group_launch_once(pf_group* g, int launch_parity) {
     return true;
 }
 
-// the work items of band b of every class at one launch parity (depth 2;
-// fused kernels only, no frozen temperature: the step clock is not read)
-bool group_launch_band(pf_group* g, int launch_parity, int b) {
+// The work items of band b of every class of one dimension at one launch parity
+// (depth 2; fused 2D kernels only, no frozen temperature: the step clock is not
+// read); pass: 1 the 3D psi pass, 2 its U pass.
+bool group_launch_band(pf_group* g, int dim, int launch_parity, int b, int pass) {
+    if (b < 0 || b >= g->n_bands) return true;
     const StepClock clk{g->clock, g->step_base, 0};
     for (const auto& c : g->classes) {
         const int lo = c.boff[b], cnt = c.boff[b + 1] - lo;
-        if (cnt <= 0) continue;
+        if (c.dim != dim || cnt <= 0) continue;
         const int grid = std::min(cnt, c.occ * num_sms());
-        const bool ok = c.dim == 3 ? launch_step3d(c.prec, c.scheme, c.bx, c.by, grid, g->st, g->work + c.w0 + lo, cnt,
-                                                   g->recs, launch_parity, clk)
-                                   : launch_step2d(c.prec, c.scheme, c.bx, grid, g->st, g->work + c.w0 + lo, cnt,
-                                                   g->recs, launch_parity, clk, c.path.var, c.path.fr);
+        const WorkItem* work = g->work + c.w0 + lo;
+        const bool ok = dim == 3 ? launch_step3d(c.prec, c.scheme, c.bx, c.by, g->st,
+                                                 Step3DArgs{work, cnt, g->recs, launch_parity, clk, c.path.fr,
+                                                            pass == 1 ? grid : 0,
+                                                            pass == 2 ? std::min(cnt, c.occ_u * num_sms()) : 0})
+                                 : launch_step2d(c.prec, c.scheme, c.bx, grid, g->st, work, cnt, g->recs, launch_parity,
+                                                 clk, c.path.var, c.path.fr);
         if (!ok) return false;
     }
     return true;
 }
 
-// two steps as one wavefront over the bands, starting at launch parity lp
+// Two steps as one wavefront over the bands, starting at launch parity lp.  3D:
+// the U pass of a band reads psi' one plane into the next band, so it follows
+// that band's psi pass, and a level-1 pass follows the last level-0 pass that
+// reads what it overwrites (psi of the band by the U pass of the band above):
+// entry (0, b) runs the psi pass of band b and the U pass of b - 1, entry (1, b)
+// the psi pass of b - 1 and the U pass of b - 2; what lags is flushed at the end.
 bool group_launch_pair(pf_group* g, int lp) {
-    const int m = 2 * g->n_bands;
+    const int nb = g->n_bands, m = 2 * nb;
     std::vector<int> level(m), band(m);
-    pf_wavefront_order(g->n_bands, level.data(), band.data(), m);
-    for (int i = 0; i < m; ++i)
-        if (!group_launch_band(g, lp ^ level[i], band[i])) return false;
-    return true;
+    pf_wavefront_order(nb, level.data(), band.data(), m);
+    auto run3 = [&](int lv, int psi_band, int u_band) {
+        return group_launch_band(g, 3, lp ^ lv, psi_band, 1) && group_launch_band(g, 3, lp ^ lv, u_band, 2);
+    };
+    for (int i = 0; i < m; ++i) {
+        const int lv = level[i], b = band[i];
+        if (!group_launch_band(g, 2, lp ^ lv, b, 0)) return false;
+        if (!(lv == 0 ? run3(0, b, b - 1) : run3(1, b - 1, b - 2))) return false;
+        if (lv == 0 && b == nb - 1 && !run3(0, -1, b)) return false;
+    }
+    return run3(1, nb - 1, nb - 2) && run3(1, -1, nb - 1);
 }
 
 }  // namespace

@@ -38,7 +38,11 @@ enum : int {
     C_UD21,      // dt D / (24 h^2): the D~_{2,1} sum's factor in the U update
     C_UD10,      // dt D / h^2
     C_UA21,      // 1 / (24 sqrt2 h^2): the anti-trapping sums', with alpha's 1/(sqrt2 dt)
-    C_UA10,      // 1 / (sqrt2 h): likewise, the <10> form normalised by |grad psi| h
+    C_UA10,      // 4 / (sqrt2 h): likewise, the <10> form normalised by 4 h |grad psi|
+    C_UD120,     // dt D / (192 h^2): the 3D sums, likewise
+    C_UD100,     // dt D / (2 h^2)
+    C_UA120,     // 1 / (192 sqrt2 h^2)
+    C_UA100,     // 2 / (sqrt2 h)
     NC
 };
 
@@ -145,14 +149,24 @@ struct StepClock {
 // frames, 2 any matrices (variant 1 only; precision 2 takes any and ignores it)
 bool launch_step2d(int prec, int scheme, int bx, int grid, cudaStream_t st, const WorkItem* work, int n_work,
                    const InstRec* recs, int launch_parity, StepClock clk, int var, int fr, int mode = 0);
-bool launch_step3d(int prec, int scheme, int bx, int by, int grid, cudaStream_t st, const WorkItem* work,
-                   int n_work, const InstRec* recs, int launch_parity, StepClock clk);
+// 3D: the psi pass, then the U pass (which reads the psi pass's psi' one plane beyond its work items), each on its own
+// grid of blocks (0: not launched); fr: 0 every cell of every instance in grain 0, 1 grain maps
+struct Step3DArgs {
+    const WorkItem* work;
+    int n_work;
+    const InstRec* recs;
+    int launch_parity;
+    StepClock clk;
+    int fr, grid_psi, grid_u;
+};
+bool launch_step3d(int prec, int scheme, int bx, int by, cudaStream_t st, const Step3DArgs& a);
 // clock += 1 (one thread)
 cudaError_t launch_tick(long long* clock, cudaStream_t st);
 // Blocks of the fused kernel that fit on one SM (0 if not compiled); var as
 // for launch_step2d
 int occupancy_step2d(int prec, int scheme, int bx, int var, int fr, int mode = 0);
-int occupancy_step3d(int prec, int scheme, int bx, int by);
+// resident blocks per SM of the two 3D passes; false if not compiled
+bool occupancy_step3d(int prec, int scheme, int bx, int by, int fr, int& psi, int& u);
 
 // Observation / initialisation kernels (observe.cu).
 struct ObsPartial {
