@@ -3,6 +3,7 @@
 // batching groups (one persistent launch per class, CUDA-graph replay).
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -107,10 +108,67 @@ int cdiv(int a, int b) { return (a + b - 1) / b; }
 // precision code of the step kernels: 0 float, 1 double, 2 compensated float pairs
 int kprec(const pf_params& p) { return p.precision == PF_F64 ? 1 : (p.precision == PF_F32C ? 2 : 0); }
 
-// capacity of the work list: the smallest tile any compiled shape produces
+// Sweep lengths of instances whose tile nobody has set.  With `per` work items a
+// unit of the GPU (2D FP32: warp schedulers; 2D FP64: SMs; 3D: SMs, items of one
+// block), a launch of sweeps of s rows takes (s + ov) row times (ov: rows
+// evaluated before the first output), each as long as one row's latency while a
+// unit holds few items and in proportion to them beyond (`fill` items keep it
+// busy), with a part of a sweep (`tail`) in which the last items run alone (half
+// of it when all items are resident at once).
+// Measured on GB300, us a step, sweeps of 32 against the choice: 128^2 FP32
+// 24.7 against 6.2, 1024^2 24.7 / 16.5, 200^2 FP64 529 / 72, 600 x 500 FP64 529 /
+// 192, 64^3 61 / 24, 96^3 74 / 43, 128^3 87 / 68; where the GPU is full anyway the
+// choice costs little (2048^2 39.0 / 39.0, 256^3 379 / 384).
+struct SweepModel {
+    int units, resident, lo, hi, by;  // resident: items a unit; lo, hi, by: the sweep lengths tried
+    double ov, fill, tail;
+};
+constexpr int GB300_SMS = 152;
+SweepModel sweep_model(const pf_params* p) {
+    if (p->dim == 3) return SweepModel{GB300_SMS, 4, 4, 24, 4, 2.5, 3.2, 0.8};
+    if (p->precision == PF_F64) return SweepModel{GB300_SMS, 8, 2, 40, 1, 2.3, 4.0, 0.3};
+    return SweepModel{4 * GB300_SMS, 4, 2, 40, 2, 2.3, 3.0, 0.5};  // (an odd sweep evaluates a row more)
+}
+// columns of work items times their extent along the sweep, per instance
+struct Strips {
+    int columns, extent;
+};
+Strips strips_of(const pf_params* p, int bx, int by) {
+    if (p->dim == 2) return Strips{cdiv(p->nx, bx - 4), p->ny};
+    return Strips{cdiv(p->nx + 1, bx - 4) * cdiv(p->ny, by - 4), p->nz};
+}
+// the cheapest sweep for instances stepped by one launch, whose items fit in max_items (0: none does)
+int pick_sweep(const SweepModel& m, const std::vector<Strips>& v, long long max_items) {
+    double best = 0.0;
+    int pick = 0;
+    for (int s = m.hi; s >= m.lo; s -= m.by) {
+        long long items = 0;
+        for (const Strips& x : v) items += (long long)x.columns * cdiv(x.extent, s);
+        if (items > max_items) continue;
+        const double per = (double)items / m.units;
+        const double cost = (s + m.ov) * std::max(1.0, (per > m.resident ? 1.0 : 0.5) * m.tail + per / m.fill);
+        if (pick == 0 || cost < best * 0.999) {
+            best = cost;
+            pick = s;
+        }
+    }
+    return pick;
+}
+// the default tile of an instance (a compensated state keeps sweeps of 32)
+struct Tile {
+    int bx, by, sweep;
+};
+Tile default_tile(const pf_params* p) {
+    Tile t = p->dim == 2 ? Tile{64, 1, 32}    // one warp per 60-column strip
+                         : Tile{34, 10, 32};  // (TX + 4, TY + 4): 30 x 6 output columns
+    if (p->precision != PF_F32C) t.sweep = pick_sweep(sweep_model(p), {strips_of(p, t.bx, t.by)}, LLONG_MAX);
+    return t;
+}
+
+// capacity of the work list: the smallest tile that pf_set_tile takes, or the default
 int max_work_items(const pf_params* p) {
-    if (p->dim == 2) return cdiv(p->nx, 60) * cdiv(p->ny, 8);
-    return cdiv(p->nx, 12) * cdiv(p->ny, 4) * cdiv(p->nz, 4);
+    if (p->dim == 3) return cdiv(p->nx, 12) * cdiv(p->ny, 4) * cdiv(p->nz, 4);
+    return std::max(cdiv(p->nx, 60) * cdiv(p->ny, 8), cdiv(p->nx, 60) * cdiv(p->ny, default_tile(p).sweep));
 }
 
 // whether d psi/dt travels between the passes in device memory: the 2D two-kernel
@@ -184,6 +242,7 @@ struct pf_sim {
     int64_t step;
     int bx, by, sweep, n_work, grid, grid_u;  // grid_u: the 3D U pass
     bool work_dirty;
+    bool auto_tile;  // the tile is the library's choice (no pf_set_tile)
     std::vector<WorkItem> work_h;
     std::vector<int> have_prev;       // per grain + 2 (index 0: pulling axis, 1: global)
     std::vector<double> prev;         // t, x, y, z per slot
@@ -192,31 +251,18 @@ struct pf_sim {
 
 namespace {
 
-void default_tile(pf_sim* s) {
-    if (s->p.dim == 2) {
-        s->bx = 64;  // one warp per 60-column strip
-        s->by = 1;
-        s->sweep = 32;
-    } else {
-        // (TX + 4, TY + 4): 30 x 6 output columns
-        s->bx = 34;
-        s->by = 10;
-        s->sweep = 32;
-    }
-}
-
-void build_work(const pf_sim* s, int inst, std::vector<WorkItem>& out) {
+void build_work(const pf_sim* s, int inst, int sweep, std::vector<WorkItem>& out) {
     const pf_params& p = s->p;
     if (p.dim == 2) {
         const int TX = s->bx - 4;
-        for (int y0 = 0; y0 < p.ny; y0 += s->sweep)
-            for (int x0 = 0; x0 < p.nx; x0 += TX) out.push_back(WorkItem{inst, x0, y0, 0, s->sweep, 0, 0, 0});
+        for (int y0 = 0; y0 < p.ny; y0 += sweep)
+            for (int x0 = 0; x0 < p.nx; x0 += TX) out.push_back(WorkItem{inst, x0, y0, 0, sweep, 0, 0, 0});
     } else {
         // a strip's outputs are the columns x0 - 1 .. x0 + TX - 2
         const int TX = s->bx - 4, TY = s->by - 4;
-        for (int z0 = 0; z0 < p.nz; z0 += s->sweep)
+        for (int z0 = 0; z0 < p.nz; z0 += sweep)
             for (int y0 = 0; y0 < p.ny; y0 += TY)
-                for (int x0 = 0; x0 < p.nx + 1; x0 += TX) out.push_back(WorkItem{inst, x0, y0, z0, s->sweep, 0, 0, 0});
+                for (int x0 = 0; x0 < p.nx + 1; x0 += TX) out.push_back(WorkItem{inst, x0, y0, z0, sweep, 0, 0, 0});
     }
 }
 
@@ -329,7 +375,7 @@ InstRec make_rec(const pf_sim* s, int parity_offset) {
 
 int upload_work(pf_sim* s) {
     s->work_h.clear();
-    build_work(s, 0, s->work_h);
+    build_work(s, 0, s->sweep, s->work_h);
     if ((int)s->work_h.size() > s->L.max_work) return PF_ERR_INVALID;
     s->n_work = (int)s->work_h.size();
     CK(cudaMemcpyAsync(s->work, s->work_h.data(), s->work_h.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, s->st));
@@ -470,7 +516,11 @@ int pf_create(const pf_params* p, void* dev_mem, size_t bytes, void* stream, pf_
     s->group = nullptr;
     s->have_prev.assign(3, 0);
     s->prev.assign(12, 0.0);
-    default_tile(s);
+    const Tile tile = default_tile(p);
+    s->bx = tile.bx;
+    s->by = tile.by;
+    s->sweep = tile.sweep;
+    s->auto_tile = true;
     int rc;
     if ((rc = upload_rot(s)) != PF_OK) { delete s; return rc; }
     cudaError_t e;
@@ -882,10 +932,10 @@ int pf_set_tile(pf_sim* s, int block_x, int block_y, int sweep) {
     if (block_x) s->bx = block_x;
     if (block_y) s->by = block_y;
     if (sweep) s->sweep = sweep;
-    bool ok = s->sweep >= 8 && s->sweep <= 1 << 20 && occupancy(s) > 0;
+    bool ok = (sweep == 0 || (sweep >= 8 && sweep <= 1 << 20)) && occupancy(s) > 0;
     if (ok) {
         std::vector<WorkItem> tmp;
-        build_work(s, 0, tmp);
+        build_work(s, 0, s->sweep, tmp);
         ok = (int)tmp.size() <= s->L.max_work;
     }
     if (!ok) {
@@ -894,6 +944,7 @@ int pf_set_tile(pf_sim* s, int block_x, int block_y, int sweep) {
         s->sweep = osw;
         return PF_ERR_INVALID;
     }
+    if (sweep) s->auto_tile = false;
     return upload_work(s);
 }
 
@@ -1095,14 +1146,40 @@ int group_rebuild(pf_group* g) {
         recs.push_back(make_rec(s, (int)((s->step ^ g->launches) & 1)));
         g->gens.push_back(s->rec_gen);
     }
+    // Sweeps: a member's own, but the 2D members of a class whose tiles nobody
+    // has set share one that suits the whole launch (a cell's bits do not depend
+    // on it); in a wavefront's bands, one of at least 8 rows.
+    std::vector<int> sweep(g->members.size());
+    for (size_t m = 0; m < g->members.size(); ++m) sweep[m] = g->members[m]->sweep;
+    auto shares = [&](int i) {
+        const pf_sim* s = g->members[i];
+        return s->auto_tile && s->p.dim == 2 && s->p.precision != PF_F32C;
+    };
+    for (size_t a = 0; a < order.size();) {
+        size_t b = a;
+        std::vector<Strips> v;
+        for (; b < order.size() && key(order[b]) == key(order[a]); ++b)
+            if (shares(order[b])) v.push_back(strips_of(&g->members[order[b]]->p, 64, 1));
+        if (!v.empty()) {
+            // other groups' launches usually fill the tail (batch.Batch)
+            SweepModel model = sweep_model(&g->members[order[a]]->p);
+            if (v.size() > 1) model.tail = 0.2;
+            const int s = g->depth == 2 ? 32 : pick_sweep(model, v, g->max_work);
+            for (; a < b; ++a)
+                if (s > 0 && shares(order[a])) sweep[order[a]] = s;
+        }
+        a = b;
+    }
     long long prev = -1;
     // depth 2 applies when no member has a frozen temperature or the
     // two-kernel form; a band must be at least two rows high (the psi halo),
     // which sweeps of at least 8 rows already guarantee
     g->wave = g->depth == 2;
-    for (const pf_sim* s : g->members)
-        if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.kernels == PF_TWO_KERNELS || (long long)g->band_sweeps * s->sweep < 2)
+    for (size_t m = 0; m < g->members.size(); ++m) {
+        const pf_sim* s = g->members[m];
+        if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.kernels == PF_TWO_KERNELS || (long long)g->band_sweeps * sweep[m] < 2)
             g->wave = false;
+    }
     g->n_bands = 0;
     std::vector<int> band_of;  // depth 2: band of every work item, in work order
     for (int i : order) {
@@ -1116,12 +1193,12 @@ int group_rebuild(pf_group* g) {
         }
         g->classes.back().path.fr = std::max(g->classes.back().path.fr, path_of(s).fr);
         const size_t first = work.size();
-        build_work(s, i, work);
+        build_work(s, i, sweep[i], work);
         g->classes.back().n = (int)work.size() - g->classes.back().w0;
         if (g->wave)
             for (size_t w = first; w < work.size(); ++w) {
                 const int c0 = s->p.dim == 2 ? work[w].y0 : work[w].z0;
-                band_of.push_back(c0 / s->sweep / g->band_sweeps);
+                band_of.push_back(c0 / sweep[i] / g->band_sweeps);
                 g->n_bands = std::max(g->n_bands, band_of.back() + 1);
             }
     }
@@ -1285,7 +1362,7 @@ int pf_group_get_depth(pf_group* g, int* depth, int* band_sweeps, int* effective
 int pf_group_work_items(const pf_sim* s) {
     if (!s) return PF_ERR_INVALID;
     std::vector<WorkItem> tmp;
-    build_work(s, 0, tmp);
+    build_work(s, 0, s->sweep, tmp);
     return (int)tmp.size();
 }
 
