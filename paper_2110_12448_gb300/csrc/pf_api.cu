@@ -126,6 +126,7 @@ struct SweepModel {
 constexpr int GB300_SMS = 152;
 SweepModel sweep_model(const pf_params* p) {
     if (p->dim == 3) return SweepModel{GB300_SMS, 4, 4, 24, 4, 2.5, 3.2, 0.8};
+    if (p->precision == PF_F32C) return SweepModel{4 * GB300_SMS, 3, 2, 56, 1, 2.3, 2.2, 0.5};
     if (p->precision == PF_F64) return SweepModel{GB300_SMS, 8, 2, 40, 1, 2.3, 4.0, 0.3};
     return SweepModel{4 * GB300_SMS, 4, 2, 40, 2, 2.3, 3.0, 0.5};  // (an odd sweep evaluates a row more)
 }
@@ -154,14 +155,14 @@ int pick_sweep(const SweepModel& m, const std::vector<Strips>& v, long long max_
     }
     return pick;
 }
-// the default tile of an instance (a compensated state keeps sweeps of 32)
+// the default tile of an instance
 struct Tile {
     int bx, by, sweep;
 };
 Tile default_tile(const pf_params* p) {
     Tile t = p->dim == 2 ? Tile{64, 1, 32}    // one warp per 60-column strip
                          : Tile{34, 10, 32};  // (TX + 4, TY + 4): 30 x 6 output columns
-    if (p->precision != PF_F32C) t.sweep = pick_sweep(sweep_model(p), {strips_of(p, t.bx, t.by)}, LLONG_MAX);
+    t.sweep = pick_sweep(sweep_model(p), {strips_of(p, t.bx, t.by)}, LLONG_MAX);
     return t;
 }
 
@@ -1153,7 +1154,7 @@ int group_rebuild(pf_group* g) {
     for (size_t m = 0; m < g->members.size(); ++m) sweep[m] = g->members[m]->sweep;
     auto shares = [&](int i) {
         const pf_sim* s = g->members[i];
-        return s->auto_tile && s->p.dim == 2 && s->p.precision != PF_F32C;
+        return s->auto_tile && s->p.dim == 2;
     };
     for (size_t a = 0; a < order.size();) {
         size_t b = a;
