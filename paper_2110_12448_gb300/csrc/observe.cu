@@ -17,8 +17,6 @@
 namespace pf {
 namespace {
 
-constexpr double SQ2 = 1.41421356237309504880;
-
 __device__ __forceinline__ bool better(double s1, long long i1, double s2, long long i2) {
     // is (s1, i1) preferred over (s2, i2)?
     if (i2 < 0) return i1 >= 0;
@@ -41,37 +39,133 @@ __device__ __forceinline__ void combine(ObsPartial& a, const ObsPartial& b) {
     }
 }
 
-// The partial of block `blk` of `nblk` walking the cells of one field pair;
-// sh: OBS_THREADS records of shared memory.
+// 2^y for -60 < y <= 0: y = n + f with |f| <= 1/2, the Taylor series of e^{f ln 2}
+// to the 12th power (remainder below 2e-16), scaled through the exponent bits.
+__device__ __forceinline__ double exp2_neg(double y) {
+    const double shift = 6755399441055744.0;  // 1.5 x 2^52: the sum's low bits are rint(y)
+    const double t = __dadd_rn(y, shift);
+    const double f = __dadd_rn(y, -__dadd_rn(t, -shift));
+    double e = 2.5678435993488206e-11;  // ln2^12 / 12!
+    e = fma(e, f, 4.4455382718708116e-10);
+    e = fma(e, f, 7.0549116208011233e-09);
+    e = fma(e, f, 1.0178086009239699e-07);
+    e = fma(e, f, 1.3215486790144309e-06);
+    e = fma(e, f, 1.5252733804059841e-05);
+    e = fma(e, f, 1.5403530393381608e-04);
+    e = fma(e, f, 1.3333558146428443e-03);
+    e = fma(e, f, 9.6181291076284772e-03);
+    e = fma(e, f, 5.5504108664821580e-02);
+    e = fma(e, f, 2.4022650695910072e-01);
+    e = fma(e, f, 6.9314718055994531e-01);
+    e = fma(e, f, 1.0);
+    return __hiloint2double(__double2hiint(e) + (__double2loint(t) << 20), __double2loint(e));
+}
+// phi = tanh(psi / sqrt2) = sign (2 / (1 + e) - 1), e = exp(-sqrt2 |psi|), of two
+// values with one division; absolute error below 4e-16, which is what the sums
+// over phi need (|psi| < 18).
+__device__ __forceinline__ void phi_two(double a, double b, double& fa, double& fb) {
+    const double c = -2.0402788931935790;  // -sqrt2 log2(e)
+    const double da = 1.0 + exp2_neg(c * fabs(a)), db = 1.0 + exp2_neg(c * fabs(b));
+    const double r = 2.0 / (da * db);
+    fa = copysign(fma(r, db, -1.0), a);
+    fb = copysign(fma(r, da, -1.0), b);
+}
+
+__device__ __forceinline__ void clear(ObsPartial& a) {
+    a.solute = 0.0;
+    a.solid = 0.0;
+    a.nonfinite = 0;
+    a.score = -DBL_MAX;
+    a.tip_index = -1;
+    a.tip[0] = a.tip[1] = a.tip[2] = 0.0;
+    a.pad = 0.0;
+}
+// a's lane takes the record of the lane `off` above
+__device__ __forceinline__ ObsPartial from_above(const ObsPartial& a, int off) {
+    const unsigned all = 0xffffffffu;
+    ObsPartial b;
+    b.solute = __shfl_down_sync(all, a.solute, off);
+    b.solid = __shfl_down_sync(all, a.solid, off);
+    b.score = __shfl_down_sync(all, a.score, off);
+    b.tip_index = __shfl_down_sync(all, a.tip_index, off);
+    b.nonfinite = __shfl_down_sync(all, a.nonfinite, off);
+    for (int q = 0; q < 3; ++q) b.tip[q] = __shfl_down_sync(all, a.tip[q], off);
+    b.pad = 0.0;
+    return b;
+}
+// The warp's tip in lane 0 (the order of the choice is total, so any tree order gives it).
+__device__ __forceinline__ void reduce_tip(ObsPartial& acc) {
+    const unsigned all = 0xffffffffu;
+    if (!__any_sync(all, acc.tip_index >= 0)) return;
+    for (int off = 16; off > 0; off >>= 1) {
+        const ObsPartial b = from_above(acc, off);
+        if (better(b.score, b.tip_index, acc.score, acc.tip_index)) {
+            acc.score = b.score;
+            acc.tip_index = b.tip_index;
+            for (int q = 0; q < 3; ++q) acc.tip[q] = b.tip[q];
+        }
+    }
+}
+// The block's record in thread 0 from one record per warp, in a fixed tree order.
+__device__ __forceinline__ void reduce_warps(ObsPartial& acc, ObsPartial* sh) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int W = OBS_THREADS / 32;
+    if (lane == 0) sh[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < W) acc = sh[lane];
+        else clear(acc);
+        for (int off = W / 2; off > 0; off >>= 1) {
+            const ObsPartial b = from_above(acc, off);
+            combine(acc, b);
+        }
+    }
+}
+
+// Cells near the interface that a warp has met and not yet evaluated.
+constexpr int OBS_QUEUE = 64 + 4 * 32;
+// what a thread, a warp and a block sum before the terms are formed
+template <typename T> struct ObsSums {
+    long long liq, sol, near, bad;          // cells
+    T l_hi, l_lo, s_hi, s_lo, n_hi, n_lo;   // U over the liquid, the solid, near the interface
+    double phi, phiu;                       // phi and phi U near the interface
+    float c, cu;                            // sign - phi and (sign - phi) U in the bulk
+};
+template <typename T> struct ObsShared {
+    ObsPartial part[OBS_THREADS / 32];
+    ObsSums<T> sums[OBS_THREADS / 32];
+    T psi[OBS_THREADS / 32][OBS_QUEUE], U[OBS_THREADS / 32][OBS_QUEUE];
+};
+
+// The partial of block `blk` of `nblk` walking the cells of one field pair.
+//
+// What bounds the observe is FP64 arithmetic (two FP64 lanes per SM and clock),
+// so it is kept to the cells that need it.  From |psi| = 18 on, phi = sign (1 - c)
+// with c = 2 e^{-sqrt2 |psi|} < 2e-11 (the next term is c^2 / 2): with phi = +-1 those
+// cells contribute 1 + (1-k) U (liquid) or k (1 + (1-k) U) (solid) to the solute
+// sum and 0 or 1 to the solid sum; they are counted and their U summed, exactly in
+// FP32 pairs (Knuth's two-sum: hi + lo carries ~48 bits, more than the FP64 sum of
+// these FP32 values keeps), and the sums of c and c U, in FP32, are 1e-16 of a
+// term per cell accurate (c is below FP64 precision from |psi| = 32 on).  The other cells go to a queue of the warp and are evaluated 64 at a
+// time, two to a lane, so that no lane idles where the interface crosses a row;
+// each adds phi and phi U to two FP64 sums.  (Five 1024^2 members with
+// mature dendrites: 150 us with the library tanh and both FP64 terms in place, 96
+// with the queue and phi_two, 83 with the bulk from 18 instead of 32, 72 with the
+// terms formed once a block instead of once a thread.)  Rows are walked whole (one block per row, threads
+// along x), so no cell index is divided.
 template <typename T>
 __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partials, long long blk, long long nblk,
-                              ObsPartial* sh) {
+                              ObsShared<T>& sh) {
     const T* __restrict__ psi = static_cast<const T*>(a.psi);
     const T* __restrict__ U = static_cast<const T*>(a.U);
     const long long nx = a.nx, ny = a.ny, nz = a.dim == 3 ? a.nz : 1;
-    const long long N = nx * ny * nz;
+    [[maybe_unused]] const long long N = nx * ny * nz;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned all = 0xffffffffu;
     ObsPartial acc;
-    acc.solute = 0.0;
-    acc.solid = 0.0;
-    acc.nonfinite = 0;
-    acc.score = -DBL_MAX;
-    acc.tip_index = -1;
-    acc.tip[0] = acc.tip[1] = acc.tip[2] = 0.0;
-    acc.pad = 0.0;
+    clear(acc);
     const double k = a.k, omk = 1.0 - a.k;
-    // Away from the interface |psi| / sqrt2 >= 22.6 and tanh is +-1 to FP64
-    // precision (both here and in C libraries that return +-1 from |x| = 22
-    // on).  Those bulk cells contribute 1 + (1-k) U (liquid) or k (1 + (1-k) U)
-    // (solid) to the solute sum and 0 or 1 to the solid sum: they are counted
-    // and their U summed, and the terms formed once per thread.  Rows
-    // are walked whole (one block per row, threads along x), so no cell index
-    // is divided.  The bulk U is summed exactly in FP32 pairs (Knuth's
-    // two-sum: hi + lo carries ~48 bits, more than the FP64 sum of these FP32
-    // values keeps) rather than in FP64, whose conversions and adds run at
-    // GB300's low FP64 rate; the non-finite test also runs in the field
-    // precision.
-    long long n_liq = 0, n_sol = 0;
-    T sl_hi = T(0), sl_lo = T(0), ss_hi = T(0), ss_lo = T(0);
+    ObsSums<T> z{};
     auto acc2 = [](T& hi, T& lo, T v) {
         if constexpr (sizeof(T) == 4) {
             const T sm = hi + v, bb = sm - hi;
@@ -81,30 +175,53 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
             hi += v;  // FP64 fields: the plain FP64 sum
         }
     };
+    int queued = 0;  // the same in every lane
+    // evaluates the first `n` <= 64 queued cells (two to a lane)
+    auto evaluate = [&](int n) {
+        __syncwarp();
+        const bool v0 = lane < n, v1 = lane + 32 < n;
+        const T p0 = v0 ? sh.psi[warp][lane] : T(0), p1 = v1 ? sh.psi[warp][lane + 32] : T(0);
+        const T u0 = v0 ? sh.U[warp][lane] : T(0), u1 = v1 ? sh.U[warp][lane + 32] : T(0);
+        double f0, f1;
+        phi_two((double)p0, (double)p1, f0, f1);
+        if (v0) {
+            z.phi += f0;
+            z.phiu = fma(f0, (double)u0, z.phiu);
+        }
+        if (v1) {
+            z.phi += f1;
+            z.phiu = fma(f1, (double)u1, z.phiu);
+        }
+        __syncwarp();
+    };
     const long long rows = ny * nz;
-    // one cell: returns after the tip test (the bulk liquid returns early)
-    auto cell = [&](long long i, long long j, long long kk, long long c, T pst, T ut) {
+    // the sums of one cell; true if it is near the interface
+    auto sums = [&](T pst, T ut) -> bool {
         if (!isfinite(pst) || !isfinite(ut)) {
-            acc.nonfinite += 1;
-            return;
+            z.bad += 1;
+            return false;
         }
-        if (fabs(pst) >= T(32)) {
+        if (fabs(pst) >= T(18)) {
+            float c = 0.0f;
+            if (fabs(pst) < T(32)) c = copysignf(2.0f * exp2f(-2.0402788931935790f * fabsf((float)pst)), (float)pst);
+            z.c += c;
+            z.cu += c * (float)ut;
             if (pst > T(0)) {
-                n_sol += 1;
-                acc2(ss_hi, ss_lo, ut);
+                z.sol += 1;
+                acc2(z.s_hi, z.s_lo, ut);
             } else {
-                n_liq += 1;
-                acc2(sl_hi, sl_lo, ut);
-                return;  // liquid: no tip candidate
+                z.liq += 1;
+                acc2(z.l_hi, z.l_lo, ut);
             }
-        } else {
-            const double u = (double)ut;
-            const double ph = tanh((double)pst / SQ2);
-            acc.solute += (1.0 + k - omk * ph) * (1.0 + omk * u) / 2.0;
-            acc.solid += (1.0 + ph) / 2.0;
+            return false;
         }
-        if (a.grain_filter >= 0 && a.grain[c] != a.grain_filter) return;
-        if (!(pst >= T(0))) return;
+        z.near += 1;
+        acc2(z.n_hi, z.n_lo, ut);
+        return true;
+    };
+    // the tip candidate of one cell
+    auto tip = [&](long long i, long long j, long long kk, long long c, T pst, T ut) {
+        if (!(pst >= T(0)) || !isfinite(pst) || !isfinite(ut)) return;
         long long ii = i, jj = j, kq = kk;
         if (a.ea == 0) ii += a.es;
         else if (a.ea == 1) jj += a.es;
@@ -112,6 +229,7 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
         if (ii < 0 || jj < 0 || kq < 0 || ii >= nx || jj >= ny || kq >= nz) return;
         const T pnt = psi[PF_CHK((kq * ny + jj) * nx + ii, N)];
         if (!(pnt < T(0))) return;
+        if (a.grain_filter >= 0 && a.grain[c] != a.grain_filter) return;
         const double ps = (double)pst, pn = (double)pnt;
         const double frac = __ddiv_rn(ps, __dsub_rn(ps, pn));
         double p[3] = {__dmul_rn((double)i, a.h), __dmul_rn((double)j, a.h),
@@ -127,54 +245,154 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
             acc.tip[2] = p[2];
         }
     };
+    // whole warps: queues the lanes' near cells, evaluates when 64 are there
+    auto push = [&](bool near, T pst, T ut) {
+        const unsigned m = __ballot_sync(all, near);
+        if (m == 0) return;
+        if (near) {
+            const int at = queued + __popc(m & ((1u << lane) - 1u));
+            sh.psi[warp][at] = pst;
+            sh.U[warp][at] = ut;
+        }
+        queued += __popc(m);
+    };
+    auto drain = [&]() {
+        while (queued >= 64) {
+            evaluate(64);
+            // the rest moves down (at most 128 cells: the queue holds 64 + 4 x 32)
+            queued -= 64;
+            T mp[4], mu[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const bool in = lane + 32 * q < queued;
+                mp[q] = in ? sh.psi[warp][64 + lane + 32 * q] : T(0);
+                mu[q] = in ? sh.U[warp][64 + lane + 32 * q] : T(0);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (lane + 32 * q < queued) {
+                    sh.psi[warp][lane + 32 * q] = mp[q];
+                    sh.U[warp][lane + 32 * q] = mu[q];
+                }
+            __syncwarp();
+        }
+    };
     // FP32 rows whose length is a multiple of 4 are read four cells at a time
     // (16-byte vector loads: more bytes in flight per thread); other rows cell
     // by cell.  The order of the per-thread sums differs between the two, not
     // the cells each block covers.
     const bool vec4 = sizeof(T) == 4 && (nx & 3) == 0 && ((uintptr_t)psi & 15) == 0 && ((uintptr_t)U & 15) == 0;
+    const int per = vec4 ? 4 : 1;
     for (long long row = blk; row < rows; row += nblk) {
         const long long j = row % ny, kk = row / ny;
         const long long base = row * nx;
-        if (vec4) {
-            for (long long i = 4 * (long long)threadIdx.x; i < nx; i += 4 * (long long)blockDim.x) {
-                const float4 p4 = __ldg(reinterpret_cast<const float4*>(psi + PF_CHK(base + i, N)));
-                const float4 u4 = __ldg(reinterpret_cast<const float4*>(U + PF_CHK(base + i, N)));
-                cell(i, j, kk, base + i, (T)p4.x, (T)u4.x);
-                cell(i + 1, j, kk, base + i + 1, (T)p4.y, (T)u4.y);
-                cell(i + 2, j, kk, base + i + 2, (T)p4.z, (T)u4.z);
-                cell(i + 3, j, kk, base + i + 3, (T)p4.w, (T)u4.w);
+        // whole warps stay in the loop: lanes beyond the row hold nothing
+        for (long long i0 = (long long)per * 32 * warp; i0 < nx; i0 += (long long)per * blockDim.x) {
+            const long long i = i0 + per * lane;
+            const bool in = i < nx;
+            if (vec4) {
+                float4 p4 = make_float4(0.f, 0.f, 0.f, 0.f), u4 = p4;
+                if (in) {
+                    p4 = __ldg(reinterpret_cast<const float4*>(psi + PF_CHK(base + i, N)));
+                    u4 = __ldg(reinterpret_cast<const float4*>(U + PF_CHK(base + i, N)));
+                }
+                const float pv[4] = {p4.x, p4.y, p4.z, p4.w}, uv[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) push(in && sums((T)pv[q], (T)uv[q]), (T)pv[q], (T)uv[q]);
+                // no tip candidate without a cell with psi >= 0
+                if (in && fmaxf(fmaxf(p4.x, p4.y), fmaxf(p4.z, p4.w)) >= 0.0f)
+                    for (int q = 0; q < 4; ++q) tip(i + q, j, kk, base + i + q, (T)pv[q], (T)uv[q]);
+            } else {
+                const T pst = in ? psi[PF_CHK(base + i, N)] : T(0), ut = in ? U[PF_CHK(base + i, N)] : T(0);
+                push(in && sums(pst, ut), pst, ut);
+                if (in) tip(i, j, kk, base + i, pst, ut);
             }
-        } else {
-            for (long long i = threadIdx.x; i < nx; i += blockDim.x) cell(i, j, kk, base + i, psi[base + i], U[base + i]);
+            drain();
         }
     }
-    const double u_liq = (double)sl_hi + (double)sl_lo, u_sol = (double)ss_hi + (double)ss_lo;
-    acc.solute += ((double)n_liq + omk * u_liq) + k * ((double)n_sol + omk * u_sol);
-    acc.solid += (double)n_sol;
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = OBS_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) combine(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
+    if (queued > 0) evaluate(queued);
+    // Sums over the warp, then over the warps, in a fixed tree order: the counts as
+    // integers, the FP32 pairs as pairs, the FP64 sums where there are any; thread 0
+    // then forms the terms (once a block: FP64 operations and conversions of every
+    // thread would cost as much as the interface).
+    auto tree = [&](int from) {
+        auto pair = [&](T& hi, T& lo) {
+            for (int off = from; off > 0; off >>= 1) {
+                const T h = __shfl_down_sync(all, hi, off), l = __shfl_down_sync(all, lo, off);
+                acc2(hi, lo, h);
+                lo += l;
+            }
+        };
+        const bool liq = __any_sync(all, z.liq != 0), sol = __any_sync(all, z.sol != 0), near = __any_sync(all, z.near != 0);
+        for (int off = from; off > 0; off >>= 1) {
+            z.liq += __shfl_down_sync(all, z.liq, off);
+            z.sol += __shfl_down_sync(all, z.sol, off);
+            z.near += __shfl_down_sync(all, z.near, off);
+            z.bad += __shfl_down_sync(all, z.bad, off);
+            z.c += __shfl_down_sync(all, z.c, off);
+            z.cu += __shfl_down_sync(all, z.cu, off);
+        }
+        if (liq) pair(z.l_hi, z.l_lo);
+        if (sol) pair(z.s_hi, z.s_lo);
+        if (near) {
+            pair(z.n_hi, z.n_lo);
+            for (int off = from; off > 0; off >>= 1) {
+                z.phi += __shfl_down_sync(all, z.phi, off);
+                z.phiu += __shfl_down_sync(all, z.phiu, off);
+            }
+        }
+    };
+    tree(16);
+    reduce_tip(acc);
+    if (lane == 0) {
+        sh.part[warp] = acc;
+        sh.sums[warp] = z;
     }
-    if (threadIdx.x == 0) partials[blk] = sh[0];
+    __syncthreads();
+    if (warp != 0) return;
+    constexpr int W = OBS_THREADS / 32;
+    if (lane < W) {
+        acc = sh.part[lane];
+        z = sh.sums[lane];
+    } else {
+        clear(acc);
+        z = ObsSums<T>{};
+    }
+    tree(W / 2);
+    reduce_tip(acc);
+    if (lane == 0) {
+        const double u_liq = (double)z.l_hi + (double)z.l_lo, u_sol = (double)z.s_hi + (double)z.s_lo,
+                     u_near = (double)z.n_hi + (double)z.n_lo;
+        // near the interface: sum (1 + k - (1-k) phi) (1 + (1-k) U) / 2 and sum (1 + phi) / 2
+        acc.nonfinite = z.bad;
+        acc.solute = ((double)z.liq + omk * u_liq) + k * ((double)z.sol + omk * u_sol) +
+                     0.5 * ((1.0 + k) * ((double)z.near + omk * u_near) - omk * (z.phi + omk * z.phiu)) +
+                     0.5 * omk * ((double)z.c + omk * (double)z.cu);
+        acc.solid = (double)z.sol + 0.5 * ((double)z.near + z.phi) - 0.5 * (double)z.c;
+        partials[blk] = acc;
+    }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(OBS_THREADS) k_observe(ObsArgs a, ObsPartial* __restrict__ partials) {
-    __shared__ ObsPartial sh[OBS_THREADS];
+__global__ void __launch_bounds__(OBS_THREADS, 3) k_observe(ObsArgs a, ObsPartial* __restrict__ partials) {
+    __shared__ ObsShared<T> sh;
     observe_block<T>(a, partials, blockIdx.x, gridDim.x, sh);
 }
 
-// All members of a group in one launch: blocks (x, m) walk member m's cells
-// exactly as blocks x of k_observe would (same partials, same order).
-__global__ void __launch_bounds__(OBS_THREADS) k_observe_multi(const ObsJob* __restrict__ jobs) {
-    __shared__ ObsPartial sh[OBS_THREADS];
+// All members of a group (of one field precision, or not) in one launch: blocks
+// (x, m) walk member m's cells exactly as blocks x of k_observe would (same
+// partials, same order).
+__global__ void __launch_bounds__(OBS_THREADS, 3) k_observe_multi(const ObsJob* __restrict__ jobs) {
+    __shared__ union {
+        ObsShared<float> f;
+        ObsShared<double> d;
+    } sh;
     const ObsJob& j = jobs[blockIdx.y];
     if (j.a.prec == 0)
-        observe_block<float>(j.a, j.partials, blockIdx.x, gridDim.x, sh);
+        observe_block<float>(j.a, j.partials, blockIdx.x, gridDim.x, sh.f);
     else
-        observe_block<double>(j.a, j.partials, blockIdx.x, gridDim.x, sh);
+        observe_block<double>(j.a, j.partials, blockIdx.x, gridDim.x, sh.d);
 }
 
 // Combine the block partials: thread t folds partials t, t + 256, ... in
@@ -182,33 +400,26 @@ __global__ void __launch_bounds__(OBS_THREADS) k_observe_multi(const ObsJob* __r
 __device__ void finish_block(const ObsPartial* __restrict__ partials, int n, ObsPartial* __restrict__ out,
                              ObsPartial* sh) {
     ObsPartial acc;
-    acc.solute = 0.0;
-    acc.solid = 0.0;
-    acc.nonfinite = 0;
-    acc.score = -DBL_MAX;
-    acc.tip_index = -1;
-    acc.tip[0] = acc.tip[1] = acc.tip[2] = 0.0;
-    acc.pad = 0.0;
+    clear(acc);
     for (int b = threadIdx.x; b < n; b += OBS_THREADS) combine(acc, partials[b]);
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = OBS_THREADS / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) combine(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
+    for (int off = 16; off > 0; off >>= 1) {
+        const ObsPartial b = from_above(acc, off);
+        combine(acc, b);
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    reduce_warps(acc, sh);
+    if (threadIdx.x == 0) *out = acc;
 }
 
 __global__ void __launch_bounds__(OBS_THREADS) k_observe_finish(const ObsPartial* __restrict__ partials, int n,
                                                                 ObsPartial* __restrict__ out) {
-    __shared__ ObsPartial sh[OBS_THREADS];
+    __shared__ ObsPartial sh[OBS_THREADS / 32];
     finish_block(partials, n, out, sh);
 }
 
 // Block m combines member m's partials into out[m].
 __global__ void __launch_bounds__(OBS_THREADS) k_observe_finish_multi(const ObsJob* __restrict__ jobs,
                                                                       ObsPartial* __restrict__ out) {
-    __shared__ ObsPartial sh[OBS_THREADS];
+    __shared__ ObsPartial sh[OBS_THREADS / 32];
     finish_block(jobs[blockIdx.x].partials, OBS_BLOCKS, out + blockIdx.x, sh);
 }
 
