@@ -228,20 +228,19 @@ template <typename T> __device__ __forceinline__ V<T> guarded_div2(V<T> f, V<T> 
 }
 
 // Resident one-warp blocks per SM that the launch bounds of the FP32 kernels
-// ask for (128 registers), and the rows that one pass of the row loop advances:
-// two with one crystal frame, so that the row state moves between registers
-// every other row only; one with per-cell frames, which spill at two (16
-// polycrystals: 136 us a step against 165).  10 x 1024^2 S-bar_21, sweeps of 38
-// rows: 65 us a step; 73 with single rows, 72 with four (the code leaves the
-// instruction cache; 99 at sweeps of 16); at single rows, 12, 14, 18 and 20
-// blocks took 82, 77, 91 and 93 us where 16 took 77.  Four columns a lane in 8
-// blocks of 240 registers: 114.  An L2 prefetch of the rows ahead: no change.
-#ifndef PF_STEP2D_BLOCKS
-#define PF_STEP2D_BLOCKS 16
-#endif
-#ifndef PF_STEP2D_ROWS
-#define PF_STEP2D_ROWS 2
-#endif
+// ask for: 17 (120 registers) where one crystal frame and no App. B magnitudes
+// are held, else 16 (128).  The row loop advances two rows per pass with one
+// crystal frame, so that the row state moves between registers every other row
+// only; one with per-cell frames, whose two copies outgrow the registers or the
+// instruction cache.  us a step, 10 x 1024^2, sweeps of 32 / 38 rows:
+//   S-bar_21  17 blocks 60.7 / 62.0, 16: 67.6 / 66.0, 18: 61.7 / 63.1
+//   S_10      17 blocks 56.7 / 57.9, 16: 64.0 / 62.5
+//   S_21      (10 x 781^2, 24 rows) 16 blocks 51.0, 17: 70.1
+// 16 polycrystals: 130.5 with 16 blocks and single rows, 161 with 17, 157 with two
+// rows.  Earlier forms of the loop: four columns a lane in 8 blocks of 240
+// registers 114 (60.7 here), three or four rows per pass 79 and 72 (68); an L2
+// prefetch of the rows ahead changes nothing.
+template <int S, int FR> constexpr int BLOCKS_F32 = FR == FR_ONE && S != S21 ? 17 : 16;
 
 // How a strip reaches its rows: WALL any strip (mirrored or wrapped columns,
 // per lane); PAIRS the whole strip, halo included, lies inside the grid and
@@ -251,7 +250,8 @@ enum : int { WALL = 0, PAIRS = 1, SINGLES = 2 };
 
 // One sweep of a work item.
 template <typename T, int S, int VAR, int FR, int MODE, int ACC>
-__device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, int launch_parity, const StepClock& clk) {
+__device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, int launch_parity, const StepClock& clk,
+                                        V<T>* park) {
     constexpr bool ISO = (S == S21 || S == SBAR21);
     constexpr bool DS = VAR == 1;   // frozen temperature / periodic x, T0 from the record
     constexpr bool T0I = VAR == 2;  // isothermal, mirror walls, T0
@@ -425,7 +425,7 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
     // one row earlier (whose results reach nothing): the loop's remainder, a third
     // copy of the row's code that rounds one product differently, never runs, and
     // a cell's bits do not depend on where a sweep ends.
-    constexpr int ROWS = sizeof(T) == 4 && FR == FR_ONE ? PF_STEP2D_ROWS : 1;
+    constexpr int ROWS = sizeof(T) == 4 && FR == FR_ONE ? 2 : 1;
     static_assert(ROWS == 1 || ROWS == 2, "rows per pass");
     const int r_end = MODE == 1 ? y1 - 1 : y1;
     int p0 = MODE == 1 ? y0 : max(y0 - 1, 0);
@@ -442,8 +442,13 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
     V2 xD0 = aD0 + east(aD0);              // a + a_E
     V2 kD = zero;                          // corner sum of row r - 1
     V2 yD = zero, ppD = zero, gD = zero;   // y+ flux, +x+y and -x+y corner fluxes of row r - 1
-    V2 aA0 = zero, xA0 = zero, kA = zero;  // the anti-trapping alpha (1 + (1-k) U) delta phi, likewise
-    V2 yA = zero, ppA = zero, gA = zero;
+    // The anti-trapping alpha (1 + (1-k) U) delta phi of row r and its sums and
+    // carries, likewise, are kept in shared memory: only rows near the interface
+    // read and write them, and the registers stay with the other rows.
+    struct AT {
+        V2 a, x, k, y, pp, g;
+    };
+    constexpr int ATN = sizeof(AT) / sizeof(V2);
     V2 phin0 = zero;                       // phi' of row r
     V2 rx = zero, ry = zero;               // S_{1,0}: |4 g h|^2 at the x+, y+ faces of row r
     // bit 0, 1: delta phi of rows r, r - 1 not exactly 0 all over the warp (clear before
@@ -617,7 +622,6 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             // Where delta phi is exactly 0 over the whole warp (bulk liquid or solid, where
             // phi = +-1 exactly) on the rows r - 1 .. r + 1, every anti-trapping flux that
             // these rows form or carry is exactly 0 and nothing of it is evaluated.
-            V2 aA1 = zero, xA1 = zero;
             bool still;
             if constexpr (T0I || MODE == 2) {
                 still = all_of(dph0, [](T d) { return d == T(0); });
@@ -625,34 +629,42 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
                 const bool s2 = DS && t0 ? dph0.x() == T(0) && dph0.y() == T(0) : phn.x() == ph.x() && phn.y() == ph.y();
                 still = __all_sync(FULL, s2);
             }
+            const bool held = (live & 7u) != 0;  // the previous row left a state
             live = live << 1 | (still ? 0u : 1u);
-            if (!still) {
-                V2 dph = dph0;
-                if constexpr (!(T0I || MODE == 2))
-                    if (!(DS && t0)) dph = phn - ph;
-                // (1 + (1-k) U) delta phi: the source of Eq. PF_b and, times 1 / (sqrt2 dt),
-                // the anti-trapping alpha
-                aA1 = fma(k_(omk), u1, c_(1.0)) * ghosts(dph);
-                xA1 = aA1 + east(aA1);
+            if (p >= ny || r < 0) {  // the ghost rows ny, -1 mirror rows ny - 1, 0
+                asm volatile("");    // a branch, not selects on every row
+                live = p >= ny ? (live & ~1u) | (live >> 1 & 1u) : (live & 1u) * 3u;
             }
-            if (p >= ny) {  // the ghost row ny mirrors row ny - 1
-                asm volatile("");  // a branch, not selects on every row
-                aA1 = aA0;
-                xA1 = xA0;
-                live = (live & ~1u) | (live >> 1 & 1u);
-            }
-            if (r < 0) {  // the ghost row -1 mirrors row 0
-                asm volatile("");
-                aA0 = aA1;
-                xA0 = xA1;
-                live = (live & 1u) * 3u | 8u;  // 8: whatever row -2 left goes
-            }
-            V2 num = aA0;
+            V2 num = zero;
             if (live & 7u) {
+                AT at{zero, zero, zero, zero, zero, zero};
+                if (held && r >= 0) {
+                    V2* q = reinterpret_cast<V2*>(&at);
+#pragma unroll
+                    for (int i = 0; i < ATN; ++i) q[i] = park[32 * i + lane];
+                }
+                V2 aA1 = zero, xA1 = zero;
+                if (!still) {
+                    V2 dph = dph0;
+                    if constexpr (!(T0I || MODE == 2))
+                        if (!(DS && t0)) dph = phn - ph;
+                    // (1 + (1-k) U) delta phi: the source of Eq. PF_b and, times 1 / (sqrt2 dt),
+                    // the anti-trapping alpha
+                    aA1 = fma(k_(omk), u1, c_(1.0)) * ghosts(dph);
+                    xA1 = aA1 + east(aA1);
+                }
+                if (p >= ny) {
+                    aA1 = at.a;
+                    xA1 = at.x;
+                }
+                if (r < 0) {
+                    at.a = aA1;
+                    at.x = xA1;
+                }
                 V2 sA;
                 if constexpr (ISO) {
                     V2 fx, fy;
-                    const V2 Ka = corner(xA0, xA1, aA0, aA1, kA, fx, fy);
+                    const V2 Ka = corner(at.x, xA1, at.a, aA1, at.k, fx, fy);
                     V2 px = fx * dm_.e, py = fy * dm, ppp = Ka * (d0_.e + dm), pg = Ka * (dm - dm_.e);
                     if constexpr (S == S21) {
                         // App. B: each anti-trapping flux divided by |grad psi| at its point, from
@@ -675,19 +687,22 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
                         ppp = guarded_div2<T>(ppp, appb_floor2<T>(mc, d0_.e + dm, ihd), hh);
                         pg = guarded_div2<T>(pg, appb_floor2<T>(mc, dm - dm_.e, ihd), hh);
                     }
-                    sA = gather(px, py, ppp, pg, yA, ppA, gA);
+                    sA = gather(px, py, ppp, pg, at.y, at.pp, at.g);
                 } else {
                     // divided by |grad psi| of the face (h and the scale of alpha are in cA)
                     auto over = [&](V2 f, V2 r2) -> V2 {
                         return select_low<T>(r2, Low<T>::face, T(0), f * rcp2(each(r2, [](T m) { return M<T>::sqrt_(m); })));
                     };
-                    const V2 px = over(c_(0.5) * xA0 * dm_.e, rx), py = over(c_(0.5) * (aA0 + aA1) * dm, ry);
-                    sA = (px - from_west(px)) + (py - yA);
-                    yA = py;
+                    const V2 px = over(c_(0.5) * at.x * dm_.e, rx), py = over(c_(0.5) * (at.a + aA1) * dm, ry);
+                    sA = (px - from_west(px)) + (py - at.y);
+                    at.y = py;
                 }
-                num = fma(k_(cA), sA, num);
-            } else if (live & 8u) {  // the last row that had any
-                kA = yA = ppA = gA = zero;
+                num = fma(k_(cA), sA, at.a);
+                at.a = aA1;
+                at.x = xA1;
+                const V2* q = reinterpret_cast<const V2*>(&at);
+#pragma unroll
+                for (int i = 0; i < ATN; ++i) park[32 * i + lane] = q[i];
             }
             if (r >= y0) store_row(U_o, r, fma(fma(k_(cD), sD, num), den, u0));
             // row p becomes row r
@@ -695,8 +710,6 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             ue0 = ue1;
             aD0 = aD1;
             xD0 = xD1;
-            aA0 = aA1;
-            xA0 = xA1;
             phin0 = phn;
             rx = rxn;
             ry = ryn;
@@ -719,9 +732,10 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
 // recomputing phase 1 (U' needs only psi^n, U^n and d psi/dt^n at the T0
 // level).
 template <typename T, int S, int VAR, int FR, int MODE>
-__global__ void __launch_bounds__(32, sizeof(T) == 4 ? PF_STEP2D_BLOCKS : 1)
+__global__ void __launch_bounds__(32, sizeof(T) == 4 ? BLOCKS_F32<S, FR> : 1)
     k_step2d(const WorkItem* __restrict__ work, int n_work, const InstRec* __restrict__ recs, int launch_parity,
              StepClock clk) {
+    __shared__ V<T> park[6 * 32];
     for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
         const WorkItem wi = work[w];
         const InstRec& rec = recs[wi.inst];
@@ -729,13 +743,13 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? PF_STEP2D_BLOCKS : 1)
             // FP64 rows take the general access: its cost disappears behind the FP64 units
             if (wi.x0 >= 2 && wi.x0 + 62 <= rec.nx) {
                 if ((rec.nx & 1) == 0)
-                    sweep2d<T, S, VAR, FR, MODE, PAIRS>(wi, rec, launch_parity, clk);
+                    sweep2d<T, S, VAR, FR, MODE, PAIRS>(wi, rec, launch_parity, clk, park);
                 else
-                    sweep2d<T, S, VAR, FR, MODE, SINGLES>(wi, rec, launch_parity, clk);
+                    sweep2d<T, S, VAR, FR, MODE, SINGLES>(wi, rec, launch_parity, clk, park);
                 continue;
             }
         }
-        sweep2d<T, S, VAR, FR, MODE, WALL>(wi, rec, launch_parity, clk);
+        sweep2d<T, S, VAR, FR, MODE, WALL>(wi, rec, launch_parity, clk, park);
     }
 }
 

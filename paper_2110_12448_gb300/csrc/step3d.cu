@@ -50,7 +50,6 @@ namespace pf {
 namespace {
 
 constexpr int SEG = 16;   // lanes of a row
-constexpr int OUTC = 30;  // output columns of a strip
 
 template <typename T> __device__ __forceinline__ T up16(T v) { return __shfl_up_sync(FULL, v, 1, SEG); }
 template <typename T> __device__ __forceinline__ T dn16(T v) { return __shfl_down_sync(FULL, v, 1, SEG); }
@@ -459,7 +458,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
     const Where<PAIRS> at(wi, rec, row);
     auto plane = [&](const T* f, int z) -> const T* { return f + (long long)PF_CHK(mirror_idx(z, nz), nz) * sxy; };
     struct Rows {
-        V2 S, C, N;
+        V2 lo, C, hi;  // rows y - 1, y, y + 1
     };
     auto read = [&](const T* f, int z) -> Rows {
         const T* P = plane(f, z);
@@ -471,7 +470,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
         auto hi = [](V2 x, V2 y) -> T { return fmax(fmax(x.x(), x.y()), fmax(y.x(), y.y())); };
         auto lo = [](V2 x, V2 y) -> T { return fmin(fmin(x.x(), x.y()), fmin(y.x(), y.y())); };
         const T B = Sat<T>::psi;
-        const T h = fmax(fmax(hi(a.S, b.S), hi(a.C, b.C)), hi(a.N, b.N)), l = fmin(fmin(lo(a.S, b.S), lo(a.C, b.C)), lo(a.N, b.N));
+        const T h = fmax(fmax(hi(a.lo, b.lo), hi(a.C, b.C)), hi(a.hi, b.hi)), l = fmin(fmin(lo(a.lo, b.lo), lo(a.C, b.C)), lo(a.hi, b.hi));
         if (__all_sync(FULL, h < -B)) return -1;
         return __all_sync(FULL, l > B) ? 1 : 0;
     };
@@ -533,11 +532,11 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
     {
         const Rows P0 = read(psi, z0 - 1), Q0 = read(psn, z0 - 1), R0 = read(Uf, z0 - 1);
         c0 = phase_of(P0, Q0);
-        b0 = beta3<T>(R0.S, R0.C, R0.N);
+        b0 = beta3<T>(R0.lo, R0.C, R0.hi);
         V2 aS, a, aN, bS, b, bN, dS, dN;
-        alphas(P0.S, Q0.S, R0.S, aS, bS, dS);
+        alphas(P0.lo, Q0.lo, R0.lo, aS, bS, dS);
         alphas(P0.C, Q0.C, R0.C, a, b, phn0);
-        alphas(P0.N, Q0.N, R0.N, aN, bN, dN);
+        alphas(P0.hi, Q0.hi, R0.hi, aN, bN, dN);
         auto first = [&](Sums3<T>& X, V2 xS, V2 x, V2 xN) {
             uniform3<T>(X, T(0));
             if constexpr (ISO) (void)weights3<T>(X, xS, x, xN);
@@ -567,7 +566,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
         asm volatile("prefetch.global.L2 [%0];" ::"l"(plane(psn, z + 4) + at.o0));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(plane(Uf, z + 4) + at.o0));
         const int c1 = phase_of(P1, Q1);
-        const Beta3<T> b1 = beta3<T>(R1.S, R1.C, R1.N);
+        const Beta3<T> b1 = beta3<T>(R1.lo, R1.C, R1.hi);
         const V2 d = b1.C - b0.C;
         V2 inc = zero;  // cD sum D + cA sum A
         V2 phn1 = k_(T(c1)), aA1 = zero;
@@ -602,9 +601,9 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
                 aS = a = aN = k_(T(1 - c1));
             } else {
                 V2 dS, dN;
-                alphas(P1.S, Q1.S, R1.S, aS, bS, dS);
+                alphas(P1.lo, Q1.lo, R1.lo, aS, bS, dS);
                 alphas(P1.C, Q1.C, R1.C, a, aA1, phn1);
-                alphas(P1.N, Q1.N, R1.N, aN, bN, dN);
+                alphas(P1.hi, Q1.hi, R1.hi, aN, bN, dN);
             }
             V2 sD;
             if constexpr (ISO) {
@@ -624,7 +623,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
                 if (live) get(&A, SUMS, ALL);
                 else clear(A);
                 const Rows P0 = read(psi, z);
-                const Beta3<T> q0 = beta3<T>(P0.S, P0.C, P0.N), q1 = beta3<T>(P1.S, P1.C, P1.N);
+                const Beta3<T> q0 = beta3<T>(P0.lo, P0.C, P0.hi), q1 = beta3<T>(P1.lo, P1.C, P1.hi);
                 const V2 dq = q1.C - q0.C;
                 V2 sA;
                 if constexpr (ISO) {
@@ -633,7 +632,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
                 } else {
                     // each face flux over |grad psi| of the face (4 h times the gradient's components)
                     const Rows Pm = read(psi, z - 1);
-                    const Beta3<T> qm = beta3<T>(Pm.S, Pm.C, Pm.N);
+                    const Beta3<T> qm = beta3<T>(Pm.lo, Pm.C, Pm.hi);
                     const V2 ez2 = c_(2.0) * (q1.C - qm.C);
                     const V2 w0 = west3(q0.e), w1 = west3(q1.e), ex0 = q0.e + w0, ey0 = q0.n - q0.s;
                     auto over = [&](V2 f, V2 gx, V2 gy, V2 gz) -> V2 {
@@ -732,7 +731,7 @@ template <typename T, int S, int TY> bool occ_t(int fr, int& psi, int& u) {
 }
 
 // Compiled tiles (block_x, block_y) = (30 + 4, TY + 4): (34, 10), and (34, 18) but for S-bar_{1,2,0} in FP64.
-template <typename T, int S> constexpr bool WIDE = sizeof(T) == 4 || S == S100;
+template <typename T, int SCH> constexpr bool WIDE = sizeof(T) == 4 || SCH == S100;
 template <typename T, int S> bool launch_s(const Step3DArgs& a, int bx, int by, cudaStream_t st) {
     if constexpr (WIDE<T, S>)
         if (bx == 34 && by == 18) return launch_t<T, S, 14>(a, st);
