@@ -1171,6 +1171,20 @@ int group_rebuild(pf_group* g) {
         }
         a = b;
     }
+    // A work list sized for longer sweeps than the defaults: the 3D members whose
+    // tiles nobody has set sweep further (their bits may depend on it).
+    auto items = [&]() {
+        long long n = 0;
+        for (size_t m = 0; m < g->members.size(); ++m) {
+            const pf_sim* s = g->members[m];
+            const Strips v = strips_of(&s->p, s->bx, s->by);
+            n += (long long)v.columns * cdiv(v.extent, sweep[m]);
+        }
+        return n;
+    };
+    for (int longer = 32; items() > g->max_work && longer <= 1 << 14; longer *= 2)
+        for (size_t m = 0; m < g->members.size(); ++m)
+            if (g->members[m]->auto_tile && g->members[m]->p.dim == 3) sweep[m] = std::max(sweep[m], longer);
     long long prev = -1;
     // depth 2 applies when no member has a frozen temperature or the
     // two-kernel form; a band must be at least two rows high (the psi halo),
