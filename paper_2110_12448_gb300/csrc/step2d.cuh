@@ -4,6 +4,36 @@
 #include "pf_internal.cuh"
 
 namespace pf {
+
+// A step kernel starts with after_previous(): its launch may begin before the
+// kernel ahead of it on the stream has ended (launch_next), and it reads and
+// writes nothing until that kernel has ended and its writes are there.  Its own
+// successor may take free slots at once where there is at most a block per SM;
+// larger grids leave that to their blocks' exit, because blocks that wait in the
+// free slots of a half-full GPU are spread unevenly (1024^2: 14.4 us a step before,
+// 12.7 so, 15.5 with a successor that waits beside it).
+constexpr int EARLY_GRID = 152;  // the SMs of GB300
+__device__ __forceinline__ void after_previous() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (gridDim.x <= EARLY_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Launches a step kernel so (programmatic stream serialisation; a capture keeps
+// it as an edge of the graph).  128^2: 6.2 -> 4.6 us a step; 200^2 FP64 72 -> 69;
+// full grids gain under 1 %.
+template <typename... P, typename... A>
+void launch_next(void (*k)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;

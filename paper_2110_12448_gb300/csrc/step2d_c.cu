@@ -571,6 +571,7 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
 template <int S>
 __global__ void __launch_bounds__(32, PF_STEP2C_BLOCKS)
     k_step2c(const WorkItem* __restrict__ work, int n_work, const InstRec* __restrict__ recs, int launch_parity) {
+    after_previous();
     for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
         const WorkItem wi = work[w];
         const InstRec& rec = recs[wi.inst];
@@ -593,7 +594,7 @@ PF_BOUNDS_READER(bounds_step2c)
 bool step2c_launch(int scheme, const Step2DArgs& a, int grid, cudaStream_t st) {
     const Kernel2C k = kernel2c(scheme);
     if (!k || a.mode != 0 || a.var != 0) return false;
-    k<<<grid, 32, 0, st>>>(a.work, a.n_work, a.recs, a.launch_parity);
+    launch_next(k, grid, 32, 0, st, a.work, a.n_work, a.recs, a.launch_parity);
     return true;
 }
 int step2c_occupancy(int scheme, int var) {

@@ -41,7 +41,7 @@ template <typename T, int S> struct Table {
 template <> bool step2d_launch<PF_REAL, PF_SCHEME>(const Step2DArgs& a, int grid, cudaStream_t st) {
     const auto k = Table<PF_REAL, PF_SCHEME>::get(a.var, a.fr, a.mode);
     if (!k) return false;
-    k<<<grid, 32, 0, st>>>(a.work, a.n_work, a.recs, a.launch_parity, a.clk);
+    launch_next(k, grid, 32, 0, st, a.work, a.n_work, a.recs, a.launch_parity, a.clk);
     return true;
 }
 template <> int step2d_occupancy<PF_REAL, PF_SCHEME>(int var, int fr, int mode) {

@@ -3,8 +3,8 @@
 //
 // Warp-per-strip design.  Each warp owns a strip of 60 output columns and
 // sweeps it row by row; lane t holds the two columns L = x0-2+2t, R = L+1
-// (lanes 0 and 31 carry the halo).  Nothing is shared between warps: there is
-// no shared memory and no block barrier.  The two columns of a lane are
+// (lanes 0 and 31 carry the halo).  Nothing is shared between warps (the little
+// shared memory holds a lane's own state) and there is no block barrier.  The two columns of a lane are
 // processed as a packed pair (FP32: the sm_100 float2 FMA/ADD/MUL
 // instructions, one issue slot for both columns).  Global traffic per step:
 // psi, U and the int16 grain read once, psi' and U' written once (float2 /
@@ -236,6 +236,8 @@ template <typename T> __device__ __forceinline__ V<T> guarded_div2(V<T> f, V<T> 
 //   S-bar_21  17 blocks 60.7 / 62.0, 16: 67.6 / 66.0, 18: 61.7 / 63.1
 //   S_10      17 blocks 56.7 / 57.9, 16: 64.0 / 62.5
 //   S_21      (10 x 781^2, 24 rows) 16 blocks 51.0, 17: 70.1
+// (17 blocks are five warps of a scheduler: 96 registers a thread, so that 20 are
+// resident.)
 // 16 polycrystals: 130.5 with 16 blocks and single rows, 161 with 17, 157 with two
 // rows.  Earlier forms of the loop: four columns a lane in 8 blocks of 240
 // registers 114 (60.7 here), three or four rows per pass 79 and 72 (68); an L2
@@ -736,6 +738,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? BLOCKS_F32<S, FR> : 1)
     k_step2d(const WorkItem* __restrict__ work, int n_work, const InstRec* __restrict__ recs, int launch_parity,
              StepClock clk) {
     __shared__ V<T> park[6 * 32];
+    after_previous();
     for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
         const WorkItem wi = work[w];
         const InstRec& rec = recs[wi.inst];

@@ -683,6 +683,7 @@ template <typename T> constexpr size_t park_bytes(int threads) { return (sizeof(
 template <typename T, int S, int TY, bool ONE>
 __global__ void __launch_bounds__(Block3<S, TY>::threads, sizeof(T) == 4 ? Block3<S, TY>::blocks : 1)
     k_psi3d(const WorkItem* __restrict__ work, int n_work, const InstRec* __restrict__ recs, int launch_parity, StepClock clk) {
+    after_previous();
     for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
         const WorkItem wi = work[w];
         const InstRec& rec = recs[wi.inst];
@@ -697,6 +698,7 @@ __global__ void __launch_bounds__(Block3<S, TY>::threads, sizeof(T) == 4 ? Block
     k_u3d(const WorkItem* __restrict__ work, int n_work, const InstRec* __restrict__ recs, int launch_parity) {
     extern __shared__ __align__(16) unsigned char smem3[];
     V<T>* park = reinterpret_cast<V<T>*>(smem3);
+    after_previous();
     for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
         const WorkItem wi = work[w];
         const InstRec& rec = recs[wi.inst];
@@ -710,10 +712,11 @@ __global__ void __launch_bounds__(Block3<S, TY>::threads, sizeof(T) == 4 ? Block
 template <typename T, int S, int TY> bool launch_t(const Step3DArgs& a, cudaStream_t st) {
     constexpr int th = Block3<S, TY>::threads;
     if (a.grid_psi > 0) {
-        if (a.fr == 0) k_psi3d<T, S, TY, true><<<a.grid_psi, th, 0, st>>>(a.work, a.n_work, a.recs, a.launch_parity, a.clk);
-        else k_psi3d<T, S, TY, false><<<a.grid_psi, th, 0, st>>>(a.work, a.n_work, a.recs, a.launch_parity, a.clk);
+        const auto k = a.fr == 0 ? k_psi3d<T, S, TY, true> : k_psi3d<T, S, TY, false>;
+        launch_next(k, a.grid_psi, th, 0, st, a.work, a.n_work, a.recs, a.launch_parity, a.clk);
     }
-    if (a.grid_u > 0) k_u3d<T, S, TY><<<a.grid_u, th, park_bytes<T>(th), st>>>(a.work, a.n_work, a.recs, a.launch_parity);
+    if (a.grid_u > 0)
+        launch_next(k_u3d<T, S, TY>, a.grid_u, th, park_bytes<T>(th), st, a.work, a.n_work, a.recs, a.launch_parity);
     return true;
 }
 template <typename T, int S, int TY> bool occ_t(int fr, int& psi, int& u) {
