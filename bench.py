@@ -64,38 +64,40 @@ def dist_env():
     return rank, world, local
 
 
-# DRAM traffic per step of the dominant kernel from an ncu capture
+# DRAM traffic per step of the step kernels from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) without cache flushes between
 # launches (--cache-control none: the lines a launch leaves dirty in L2 are
 # written back during the next one, as in a live run), valid only while the
-# kernel source is byte-identical to the one captured (sha256 of the .cu file)
-# and the launch uses the captured tile (block x, block y, sweep).
+# kernel source is byte-identical to the one captured (sha256 of the file)
+# and the launch uses the captured block shape (block x, block y).
 TRAFFIC = {
-    # one step of the orientation sweep (10 x 1024^2, tile 64 x 1 x 38): the two
+    # one step of the orientation sweep (10 x 1024^2, tile 64 x 1 x 32): the two
     # k_step2d<float, S-bar_21> launches of the two five-instance groups, summed (ncu runs them one
     # after the other, so each group's half of the state partly stays in L2)
-    "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d.cu", "tile": [64, 1, 38],
-                "sha256": "51b2245cc8536307702969be51cd8ebcc4eef9819cb65035bf04650382af4634", "bytes": 103638016},
-    # one k_step3d<float, S-bar_120, 30, 6> launch of the 256^3 free dendrite (tile 34 x 10 x 52)
-    "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 52],
-                   "sha256": "1f5d22af251dade05882fb4be57c4fe582caa7ec964125d0cab5048c80b10939", "bytes": 265664000},
+    "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d_kernel.cuh", "tile": [64, 1, 32],
+                "sha256": "098f4139e44e03eeb712f0d5416d29ffa2525db1fff24bc448fffad75246b895", "bytes": 97869824},
+    # one step of the 256^3 free dendrite (tile 34 x 10 x 26): the k_psi3d<float, S-bar_120> launch
+    # (217 MB) and the k_u3d launch (266 MB), summed
+    "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 26],
+                   "sha256": "e5d268a005ad5a36825bf9869cb714f09eaa41a4183e54e2f889451aeacb5a48", "bytes": 482729728},
 }
 
 
-# FP32 floating-point operations per cell update of the dominant kernel, from
-# an ncu capture of one launch: FADD + FMUL + 2 FFMA + 2 (FADD2 + FMUL2) +
+# FP32 floating-point operations per cell update of the step kernels, from an
+# ncu capture of one step: FADD + FMUL + 2 FFMA + 2 (FADD2 + FMUL2) +
 # 4 FFMA2 thread instructions (sm__sass_thread_inst_executed_op_*_pred_on)
-# over the launch's cell updates; like TRAFFIC, valid only while the kernel
+# over the step's cell updates; like TRAFFIC, valid only while the kernel
 # source is byte-identical to the one captured.  The FP32 peak is the unit
 # count at the maximum clock: 152 SMs x 128 FP32 lanes x 2 (FMA) x 2.07 GHz.
-# (3D: executed per output cell, including the ring-1 recompute of the tile.)
+# (Executed per output cell, including the columns and rows a warp recomputes
+# at the rim of its strip: 64 columns for 60 outputs in 2D, 32 for 30 in 3D.)
 FLOPS = {
-    # k_step2d<float, S-bar_21> launch of the orientation sweep (10 x 1024^2, tile 64 x 1 x 38)
-    "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d.cu", "tile": [64, 1, 38],
-                "sha256": "51b2245cc8536307702969be51cd8ebcc4eef9819cb65035bf04650382af4634", "flop_per_cell": 261.2},
-    # k_step3d<float, S-bar_120, 30, 6> launch of the 256^3 free dendrite (tile 34 x 10 x 52)
-    "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 52],
-                   "sha256": "1f5d22af251dade05882fb4be57c4fe582caa7ec964125d0cab5048c80b10939", "flop_per_cell": 1100.6},
+    # the two k_step2d<float, S-bar_21> launches of the orientation sweep (10 x 1024^2, tile 64 x 1 x 32)
+    "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d_kernel.cuh", "tile": [64, 1, 32],
+                "sha256": "098f4139e44e03eeb712f0d5416d29ffa2525db1fff24bc448fffad75246b895", "flop_per_cell": 200.9},
+    # k_psi3d<float, S-bar_120> + k_u3d launches of the 256^3 free dendrite (tile 34 x 10 x 26)
+    "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 26],
+                   "sha256": "e5d268a005ad5a36825bf9869cb714f09eaa41a4183e54e2f889451aeacb5a48", "flop_per_cell": 502.4},
 }
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
@@ -331,7 +333,6 @@ def fp64_plain(stream, n=200, steps=2000):
     from paper_2110_12448_gb300 import synth
     w = synth.free_dendrite_2d(n)
     s = N.Sim.from_workload(w, "f64", stream=stream)
-    s.set_tile(64, 1, 16)
     s.step(10)
     a = torch.cuda.Event(enable_timing=True)
     b = torch.cuda.Event(enable_timing=True)
@@ -880,12 +881,14 @@ def run_native(args):
                  "isotherm_y": round(ws[0].yT + DS_VP * t_now, 4),
                  "delta": [round(tips[0] - v, 4) for v in tips], "at_step": sims[0].steps_done}
 
-    # roofline of the fused step kernel: algorithmic bytes per launch / mean launch time
+    # roofline of the step's kernels: algorithmic bytes per step / mean time per step
     peak, peak_kind = peaks()
     bpc = bytes_per_cell(ws, args.precision, two=args.kernels == "two")
     achieved = cells * bpc / (kern_ms / n_launch / 1e3) / 1e9
     tname = {"f32": "float", "f64": "double", "f32c": "float, compensated state"}[args.precision]
-    kname = ("k_step2d" if ws[0].dim == 2 else "k_step3d") + f"<{tname},{args.scheme}>"
+    targs = f"<{tname},{args.scheme}>"
+    kname = f"k_psi3d{targs} + k_u3d{targs}" if ws[0].dim == 3 else \
+        ("k_step2c" if args.precision == "f32c" else "k_step2d") + targs
     if args.kernels == "two":
         kname += " psi pass + U pass (two-kernel form, T0)"
     elif args.time_level == "t0":
@@ -1006,8 +1009,10 @@ def run_native(args):
                                         "over": f"{len(per_step)} single steps of the whole batch after the timed "
                                                 f"region, each launched directly with its own events"},
                 "tile": list(tile) if tile else None,
-                # a depth-2 step is one launch per band (one class per group here)
-                "gpu_launches": (n_launch * (autotune.bands(ws, tile) if tile else 1) + 2 * n_observe)
+                # a depth-2 step is one launch per band (one class per group here); a 3D step and the
+                # two-kernel form are two kernels
+                "gpu_launches": (n_launch * (autotune.bands(ws, tile) if tile else 1)
+                                 * (2 if ws[0].dim == 3 or args.kernels == "two" else 1) + 2 * n_observe)
                                 * len(batch.groups)}
         if tune_times:
             # temporal-blocking depth as the autotuner raced it (ms per step of the batch)

@@ -86,8 +86,9 @@ enum { PF_ISOTHERMAL = 0, PF_FROZEN_GRADIENT = 1 };
  *        (conserves the solute to O(dt) over a fixed time). */
 enum { PF_T1 = 0, PF_T0 = 1 };
 /* Kernels of a step (Sec. 3.3.1 describes two, a psi kernel then a U kernel):
- * PF_FUSED: one kernel per step, psi' and the U update from the same pass
- *   (d psi/dt stays on chip);
+ * PF_FUSED: in 2D one kernel per step, psi' and the U update from the same
+ *   pass (d psi/dt stays on chip); in 3D a psi pass and a U pass that reads
+ *   psi and psi' back (with PF_T0 also d psi/dt, one more field);
  * PF_TWO_KERNELS: the psi kernel writes psi' and d psi/dt to device memory,
  *   then the U kernel reads d psi/dt back (2D, PF_T0 time level, PF_F32 or
  *   PF_F64).  Same arithmetic as the fused T0 step; it costs the extra
@@ -206,7 +207,7 @@ int pf_set_grain_index(pf_sim* s, const int16_t* host_grain);
 int pf_get_grain_index(pf_sim* s, int16_t* host_grain);
 
 /* Advance n >= 0 explicit Euler steps, queued asynchronously on the stream
- * (one fused kernel launch per step). */
+ * (one kernel launch per step in 2D, a psi pass and a U pass in 3D). */
 int pf_step(pf_sim* s, int64_t n);
 
 /* Synchronise the stream and observe grain g (0 <= g < n_grains) or, with
@@ -284,13 +285,16 @@ int pf_shift_frame(pf_sim* s, int rows);
  * the int16 grain map; valid until the next pf_step / pf_group_step. */
 int pf_device_fields(pf_sim* s, void** psi, void** U, void** grain);
 
-/* Tile shape of the fused kernel (cells per block along x, and the number
- * of rows (2D) or planes (3D) a block sweeps); 0 keeps the current value.
- * Used by the autotuner.  block_x must be one of the compiled widths. */
+/* Tile shape of the step: the widths along x and y (2D: 64 x 1 columns of a
+ * warp; 3D: a block shape of the documented list) and the number of rows (2D)
+ * or planes (3D) one work item sweeps; 0 keeps the current value.  Until a
+ * sweep is set here the library chooses it from the grid (and, in a group,
+ * from all members), and pf_get_tile reports its choice.  In 2D
+ * the results do not depend on the sweep.  Used by the autotuner. */
 int pf_set_tile(pf_sim* s, int block_x, int block_y, int sweep);
 int pf_get_tile(pf_sim* s, int* block_x, int* block_y, int* sweep);
 /* Work units of the current tile that are resident on the device at once
- * (warps in 2D, blocks in 3D).  A persistent launch runs min(work items,
+ * (warps in 2D, blocks of the psi pass in 3D).  A persistent launch runs min(work items,
  * this) units, so a work list just below a whole multiple of it balances
  * best; the autotuner picks sweep lengths from it.  Returns the count (> 0)
  * or a negative PF_ERR_* code; needs a current CUDA device. */
@@ -389,7 +393,8 @@ int pf_group_size(const pf_group* g);
  * are bit-identical.  A group whose members include a frozen temperature (one
  * step clock per launch) or a two-kernel member (its U pass needs the psi
  * pass of the neighbouring bands) steps at depth 1; pf_group_get_depth
- * reports the depth in effect.  An odd step
+ * reports the depth in effect.  In 3D the U pass of a band follows the psi
+ * pass of the next band, one band later than above, for the same reason.  An odd step
  * count ends with one depth-1 step.  depth outside {1, 2} or band_sweeps < 1
  * is PF_ERR_INVALID; the setting holds across membership changes. */
 int pf_group_set_depth(pf_group* g, int depth, int band_sweeps);
