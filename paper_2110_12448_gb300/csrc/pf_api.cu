@@ -119,6 +119,7 @@ int kprec(const pf_params& p) { return p.precision == PF_F64 ? 1 : (p.precision 
 // 24.7 against 6.2, 1024^2 24.7 / 16.5, 200^2 FP64 529 / 72, 600 x 500 FP64 529 /
 // 192, 64^3 61 / 24, 96^3 74 / 43, 128^3 87 / 68; where the GPU is full anyway the
 // choice costs little (2048^2 39.0 / 39.0, 256^3 379 / 384).
+// (Since then launches overlap, step2d.cuh: 128^2 4.6, 1024^2 12.7, 200^2 FP64 69.)
 struct SweepModel {
     int units, resident, lo, hi, by;  // resident: items a unit; lo, hi, by: the sweep lengths tried
     double ov, fill, tail;
