@@ -102,41 +102,6 @@ template <typename T> struct Low {
     static constexpr T face = T(16) * Guard<T>::v, centre = T(4) * Guard<T>::v;
 };
 
-// FP64 divisions cost a dozen FP64 instructions each at GB300's low FP64
-// rate: the denominators of one column share one (1/a = b / (a b)).  FP32
-// takes the single-instruction estimates.
-template <typename T> __device__ __forceinline__ void inv_each(V<T>& a, V<T>& b, V<T>& c) {
-    if constexpr (sizeof(T) == 8) {
-        const V<T> t = a * b;
-        const V<T> q = rcp2(t * c);
-        const V<T> u = q * c;
-        c = q * t;
-        const V<T> ia = u * b;
-        b = u * a;
-        a = ia;
-    } else {
-        a = rcp2(a);
-        b = rcp2(b);
-        c = rcp2(c);
-    }
-}
-template <typename T> __device__ __forceinline__ void inv_each(V<T>& a, V<T>& b) {
-    if constexpr (sizeof(T) == 8) {
-        const V<T> q = rcp2(a * b);
-        const V<T> ia = q * b;
-        b = q * a;
-        a = ia;
-    } else {
-        a = rcp2(a);
-        b = rcp2(b);
-    }
-}
-// squared lengths that enter a division, with the columns below the guard
-// replaced where the division is shared (the guard's select discards them)
-template <typename T> __device__ __forceinline__ V<T> guarded(V<T> r2, T low) {
-    if constexpr (sizeof(T) == 8) return each(r2, [=](T r) { return r < low ? T(1) : r; });
-    return r2;
-}
 template <typename T>
 __device__ __forceinline__ V<T> select_low(V<T> r2, T low, T other, V<T> v) {
     return each(r2, v, [=](T r, T x) { return r < low ? other : x; });
@@ -465,7 +430,7 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
         if constexpr (FR != FR_ONE) set_frame(nG);
         const V2 gx = dm_.ex + d0_.ex, gn = c_(4.0) * dm;
         const V2 r2 = fma(gx, gx, gn * gn);
-        Yc = face_flux<T, FR>(gx, gn, r2, rcp2(guarded<T>(r2, Low<T>::face)), F, an, false);
+        Yc = face_flux<T, FR>(gx, gn, r2, rcp2(r2), F, an, false);
     }
 
 #pragma unroll ROWS
@@ -510,8 +475,7 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             const V2 rX = fma(gxX, gxX, gyX * gyX);
             const V2 rY = fma(gxY, gxY, gyY * gyY);
             const V2 rC = fma(d0_.ex, d0_.ex, ey * ey);
-            V2 iX = guarded<T>(rX, Low<T>::face), iY = guarded<T>(rY, Low<T>::face), iC = guarded<T>(rC, Low<T>::centre);
-            if constexpr (FR != FR_ANY) inv_each(iX, iY, iC);
+            const V2 iX = rcp2(rX), iY = rcp2(rY), iC = rcp2(rC);
             const V2 Xp = face_flux<T, FR>(gxX, gyX, rX, iX, F, an, true);
             const V2 Yp = face_flux<T, FR>(gxY, gyY, rY, iY, F, an, false);
             // x- faces: from the left column; recomputed across grain boundaries.
@@ -525,13 +489,13 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
                     // (W + C)(p+1) - (W + C)(p-1) = 2 ey - (C - W)(p+1) + (C - W)(p-1)
                     const V2 gyW = ey2 - ((dp_.e - dp_.sx) - (dm_.e - dm_.sx));
                     const V2 r2 = fma(gxW, gxW, gyW * gyW);
-                    const V2 q = face_flux<T, FR>(gxW, gyW, r2, rcp2(guarded<T>(r2, Low<T>::face)), F, an, true);
+                    const V2 q = face_flux<T, FR>(gxW, gyW, r2, rcp2(r2), F, an, true);
                     Xm = mk(bL ? q.x() : Xm.x(), bR ? q.y() : Xm.y());
                 }
                 if (__any_sync(FULL, moved)) {
                     const V2 gx = dm_.ex + d0_.ex, gn = c_(4.0) * dm;
                     const V2 r2 = fma(gx, gx, gn * gn);
-                    const V2 q = face_flux<T, FR>(gx, gn, r2, rcp2(guarded<T>(r2, Low<T>::face)), F, an, false);
+                    const V2 q = face_flux<T, FR>(gx, gn, r2, rcp2(r2), F, an, false);
                     Ym = mk(g_lo(gf) != g_lo(g1) ? q.x() : Ym.x(), g_hi(gf) != g_hi(g1) ? q.y() : Ym.y());
                 }
                 gf = g1;
@@ -553,7 +517,6 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
                 G = c_(-1.41421356237309504880 / 4.0) * rC;
             }
             const V2 as = select_low<T>(rC, Low<T>::centre, T(1), aniso_as<T, FR>(d0_.ex, ey, iC, F, an));
-            V2 a2 = as * as;
             V2 uc = u1;      // F2 of Eq. PF_a
             T iF1 = T(1);    // 1 / F1
             if (DS) {
@@ -564,8 +527,8 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             // sqrt2 [phi - lambda (1 - phi) (1 + phi) F2]
             const V2 src = fma(aD1 * fma(k_(-lam2), ph, k_(-lam2)), uc, k_(sq) * ph);
             const V2 E = (L + N) + src;
-            inv_each(a2, den);
-            V2 rate = fma(ph, G, E * a2);
+            den = rcp2(den);
+            V2 rate = fma(ph, G, E * rcp2(as * as));
             if (DS) rate = rate * k_(iF1);
             const V2 psin = fma(k_(dtl), rate, C0);
             if constexpr (T0I) {
