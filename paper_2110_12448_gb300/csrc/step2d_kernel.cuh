@@ -244,13 +244,19 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
     const Aniso<T> an(cst[C_EPS], ISO ? T(1.5) : T(0.25));
     const bool per = DS && rec.bcx != 0;
     const bool t0 = T0I || (DS && rec.tlevel != 0);  // T0 time level
-    // frozen temperature: zeta at row p = zeta_y0 + (p - y0) zA (Eqs. Thermal_F1/_F2);
-    // the DS variant applies it branch-free (zA = zB = zC = 0 gives zeta = 0, F1 = 1)
-    T zeta_y0 = T(0), zA = T(0);
+    // Frozen temperature: zeta at row p = p zA - (zB + n zC) (Eqs. Thermal_F1/_F2) from
+    // the row's index alone, so that it does not depend on where a sweep begins; both
+    // constants with what their rounding to the field precision leaves (FP32: within an
+    // ulp of zeta, however large the two terms are).  The DS variant applies it
+    // branch-free (zA = zB = zC = 0 gives zeta = 0, F1 = 1).
+    T zA = T(0), zAl = T(0), z0 = T(0), z0l = T(0);
     if (DS) {
         const long long n = clk.clock ? clk.base[wi.inst] + *clk.clock : clk.step;
-        zeta_y0 = (T)((double)wi.y0 * rec.zA - rec.zB - (double)n * rec.zC);
+        const double b = -::fma((double)n, rec.zC, rec.zB);
         zA = (T)rec.zA;
+        zAl = (T)(rec.zA - (double)zA);
+        z0 = (T)b;
+        z0l = (T)(b - (double)z0);
     }
 
     const int x0 = wi.x0, y0 = wi.y0;
@@ -520,9 +526,10 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             V2 uc = u1;      // F2 of Eq. PF_a
             T iF1 = T(1);    // 1 / F1
             if (DS) {
-                const T z = zeta_y0 + T(p - y0) * zA;
+                T z = ::fma(T(p), zA, z0);
+                if constexpr (sizeof(T) == 4) z += ::fma(T(p), zAl, z0l);
                 uc = uc + k_(z);
-                iF1 = M<T>::rcp(T(1) - omk * z);
+                iF1 = M<T>::rcp(::fma(-omk, z, T(1)));
             }
             // sqrt2 [phi - lambda (1 - phi) (1 + phi) F2]
             const V2 src = fma(aD1 * fma(k_(-lam2), ph, k_(-lam2)), uc, k_(sq) * ph);
