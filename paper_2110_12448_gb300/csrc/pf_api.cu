@@ -1101,7 +1101,7 @@ struct pf_group {
     bool dirty;
     struct Cls {
         int dim, scheme, prec, bx, by, w0, n, grid;
-        Path path; // 2D kernel: variant and frames (the most general of the members')
+        Path path; // 2D kernel: variant and frames (per-cell frames if a member has them)
         bool two;  // two-kernel form: the psi pass, then the U pass
         int occ, occ_u;  // resident units per SM (occ_u: the 3D U pass)
         std::vector<int> boff;  // depth 2: work items of band b are [w0 + boff[b], w0 + boff[b + 1])
@@ -1137,7 +1137,9 @@ int group_rebuild(pf_group* g) {
     for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
     auto key = [&](int i) {
         const pf_sim* s = g->members[i];
-        return ((long long)s->p.kernels << 52) | ((long long)path_of(s).var << 48) | ((long long)s->p.dim << 40) |
+        const Path k = path_of(s);  // any matrices: a class of their own, the others' arithmetic is not theirs
+        return ((long long)s->p.kernels << 52) | ((long long)(k.fr == 2) << 50) | ((long long)k.var << 48) |
+               ((long long)s->p.dim << 40) |
                ((long long)s->p.scheme << 32) |
                ((long long)s->p.precision << 24) | ((long long)s->bx << 12) | (long long)s->by;
     };
