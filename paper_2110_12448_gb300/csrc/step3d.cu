@@ -44,6 +44,8 @@
 // What bounds them (256^3, S-bar_{1,2,0}): the psi pass instruction issue and the
 // FMA pipe (195 warp instructions per 60 cells, 115 of them packed arithmetic, 54 %
 // of the issue slots with 12 warps per SM), the U pass the latency of its rows.
+#include <cfloat>
+
 #include "step2d.cuh"
 
 namespace pf {
@@ -67,6 +69,23 @@ template <typename T> struct Frame3 {
 template <typename T> struct Sat;
 template <> struct Sat<float> { static constexpr float psi = 14.0f; };
 template <> struct Sat<double> { static constexpr double psi = 32.0; };
+
+// max and min that return NaN where an operand is one
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float min_nan(float a, float b) {
+    float r;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ double max_nan(double a, double b) { return a > b || isnan(a) ? a : b; }
+__device__ __forceinline__ double min_nan(double a, double b) { return a < b || isnan(a) ? a : b; }
+template <typename T> struct Largest;
+template <> struct Largest<float> { static constexpr float v = FLT_MAX; };
+template <> struct Largest<double> { static constexpr double v = DBL_MAX; };
 
 // Component `ax` of (J - g), J = d(a_s^2 |g|^2 / 2)/dg, times `scale`, for
 // gradients times 4 h in the lanes' frames: with c = R^T g, t_p = c_p^2, s_p =
@@ -464,15 +483,24 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
         const T* P = plane(f, z);
         return Rows{at.template load<T>(P, at.oS), at.template load<T>(P, at.o0), at.template load<T>(P, at.oN)};
     };
-    // phi of every cell the warp reads of a plane: -1 or 1 exactly, before and (T1) after the step; else 0
-    auto phase_of = [&](const Rows& a, const Rows& q) -> int {
+    // phi of every cell the warp reads of a plane: -1 or 1 exactly, before and (T1) after the step; else 0.
+    // A NaN is in neither phase, nor is a plane whose d psi/dt (T0) or, where phi = 1, U is not finite:
+    // there the products with alphas of 0 are evaluated, so that NaN and infinities reach U' as they would.
+    auto phase_of = [&](const Rows& a, const Rows& q, const Rows& u) -> int {
         const Rows b = t0 ? a : q;
-        auto hi = [](V2 x, V2 y) -> T { return fmax(fmax(x.x(), x.y()), fmax(y.x(), y.y())); };
-        auto lo = [](V2 x, V2 y) -> T { return fmin(fmin(x.x(), x.y()), fmin(y.x(), y.y())); };
+        auto hi = [](V2 x, V2 y) -> T { return max_nan(max_nan(x.x(), x.y()), max_nan(y.x(), y.y())); };
+        auto lo = [](V2 x, V2 y) -> T { return min_nan(min_nan(x.x(), x.y()), min_nan(y.x(), y.y())); };
+        auto finite = [](const Rows& r) -> bool {
+            T m = max_nan(fabs(r.C.x()), fabs(r.C.y()));
+            m = max_nan(m, max_nan(fabs(r.lo.x()), fabs(r.lo.y())));
+            return max_nan(m, max_nan(fabs(r.hi.x()), fabs(r.hi.y()))) <= Largest<T>::v;
+        };
         const T B = Sat<T>::psi;
-        const T h = fmax(fmax(hi(a.lo, b.lo), hi(a.C, b.C)), hi(a.hi, b.hi)), l = fmin(fmin(lo(a.lo, b.lo), lo(a.C, b.C)), lo(a.hi, b.hi));
-        if (__all_sync(FULL, h < -B)) return -1;
-        return __all_sync(FULL, l > B) ? 1 : 0;
+        const T h = max_nan(max_nan(hi(a.lo, b.lo), hi(a.C, b.C)), hi(a.hi, b.hi)),
+                l = min_nan(min_nan(lo(a.lo, b.lo), lo(a.C, b.C)), lo(a.hi, b.hi));
+        const bool rate = !t0 || finite(q);
+        if (__all_sync(FULL, h < -B && rate)) return -1;
+        return __all_sync(FULL, l > B && rate && finite(u)) ? 1 : 0;
     };
     auto phi = [](V2 p) -> V2 {
         return each3(p, [](T x) {
@@ -531,7 +559,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
     unsigned live = 0;           // bit 0: A's state is in use (in shared memory)
     {
         const Rows P0 = read(psi, z0 - 1), Q0 = read(psn, z0 - 1), R0 = read(Uf, z0 - 1);
-        c0 = phase_of(P0, Q0);
+        c0 = phase_of(P0, Q0, R0);
         b0 = beta3<T>(R0.lo, R0.C, R0.hi);
         V2 aS, a, aN, bS, b, bN, dS, dN;
         alphas(P0.lo, Q0.lo, R0.lo, aS, bS, dS);
@@ -565,7 +593,7 @@ __device__ __forceinline__ void u_sweep(const WorkItem& wi, const InstRec& rec, 
         asm volatile("prefetch.global.L2 [%0];" ::"l"(plane(psi, z + 4) + at.o0));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(plane(psn, z + 4) + at.o0));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(plane(Uf, z + 4) + at.o0));
-        const int c1 = phase_of(P1, Q1);
+        const int c1 = phase_of(P1, Q1, R1);
         const Beta3<T> b1 = beta3<T>(R1.lo, R1.C, R1.hi);
         const V2 d = b1.C - b0.C;
         V2 inc = zero;  // cD sum D + cA sum A
