@@ -11,6 +11,8 @@
 // of the double-float arithmetic (the exponential, two divisions, the coupling
 // term) forms nothing but them: a row whose |psi| exceeds FAR all over the warp
 // takes the constants (10 x 1024^2: 366 -> 260 us a step).
+#include <cfloat>
+
 #include "step2d.cuh"
 #include "step2d_launch.cuh"
 
@@ -211,9 +213,11 @@ __device__ __forceinline__ D2 dexp_neg(D2 x) {
 }
 
 
-// |psi| from which phi = +-1 - O(e^{-sqrt2 |psi|} = 2e-15), 1 - phi^2 = 0 and delta
-// phi = 0 change the psi rate by less than 1e-13, below the lo half's resolution
-// of psi there (1.1e-13 at 24) once multiplied by dt < 0.1.
+// |psi| from which the psi rate takes phi = +-1 and no coupling term.  What that
+// leaves out of dt times the rate, 4 e^{-sqrt2 24} = 7.3e-15 times sqrt2 lambda dt |U|
+// (and a quarter of it times sqrt2 dt (1 + |grad psi|^2)), is below 2.1e-14 while
+// lambda dt |U| <= 2, less than half a unit in the last place of the lo half of such a
+// psi (2.8e-14); rows with a larger U, or one that is not finite, are evaluated in full.
 constexpr float FAR = 24.0f;
 
 // Resident one-warp blocks per SM asked for: 168 registers a lane and twelve
@@ -254,6 +258,7 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
     const float kk = cst[C_K], omk = cst[C_OMK], eps = cst[C_EPS], lam = cst[C_LAM], Dc = cst[C_D];
     const float ih2 = cst[C_IH2], i6h2 = cst[C_I6H2];
     const float isq2dt = cst[C_ISQ2DT];
+    const float u_far = fminf(2.0f / (lam * dt), FLT_MAX);
     const bool one = rec.one_grain != 0;  // every cell in grain 0
     const int x0 = wi.x0, y0 = wi.y0;
     const int y1 = min(y0 + wi.ext, ny);
@@ -408,7 +413,8 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
         const V2 w = aniso_w2(ex * k_(ih_half), ey * k_(ih_half), RR, eps, hh);
         const D2 ad = dadd(kA0, d2f(w));
         const bool nL = C0.x() < 0.0f, nR = C0.y() < 0.0f;
-        const bool far = __all_sync(FULL, fabsf(C0.x()) > FAR && fabsf(C0.y()) > FAR);
+        const bool far = __all_sync(FULL, fabsf(C0.x()) > FAR && fabsf(C0.y()) > FAR && fabsf(U1.C.x()) <= u_far &&
+                                              fabsf(U1.C.y()) <= u_far);
         V2 ph, dph = zero;
         D2 srcd, phG;  // sqrt2 (phi - lambda (1 - phi^2) U) and sqrt2 phi
         if (far) {
@@ -437,6 +443,7 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
         const D2 s1 = two_sum(C0, d.h);
         const D2 s2 = fast_two_sum(s1.h, s1.l + (cl + d.l));
         if (!far) dph = mk(dphi_acc(ph.x(), d.h.x()), dphi_acc(ph.y(), d.h.y()));
+        else dph = d.h * k_(0.0f);  // 0, but NaN where the rate is not finite
         V2 phn = ph + dph;
         if (p >= y0 && p < y1) {
             store_row(psi_o, p, s2.h);
@@ -446,7 +453,7 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
         // ---------------- alphas of row p ----------------
         const Tri AD1 = tri(k_(1.0f) - ph);
         // delta phi row exactly 0 over the whole warp: bulk liquid or solid
-        const bool still = far || __all_sync(FULL, dph.x() == 0.0f && dph.y() == 0.0f);
+        const bool still = __all_sync(FULL, dph.x() == 0.0f && dph.y() == 0.0f);
         live = live << 1 | (still ? 0u : 1u);
         Tri AA1{zero, zero, zero};
         V2 src1 = zero;
