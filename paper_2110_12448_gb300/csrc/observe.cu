@@ -39,7 +39,7 @@ __device__ __forceinline__ void combine(ObsPartial& a, const ObsPartial& b) {
     }
 }
 
-// 2^y for -60 < y <= 0: y = n + f with |f| <= 1/2, the Taylor series of e^{f ln 2}
+// 2^y for -1000 < y <= 0: y = n + f with |f| <= 1/2, the Taylor series of e^{f ln 2}
 // to the 12th power (remainder below 2e-16), scaled through the exponent bits.
 __device__ __forceinline__ double exp2_neg(double y) {
     const double shift = 6755399441055744.0;  // 1.5 x 2^52: the sum's low bits are rint(y)
@@ -62,7 +62,7 @@ __device__ __forceinline__ double exp2_neg(double y) {
 }
 // phi = tanh(psi / sqrt2) = sign (2 / (1 + e) - 1), e = exp(-sqrt2 |psi|), of two
 // values with one division; absolute error below 4e-16, which is what the sums
-// over phi need (|psi| < 18).
+// over phi need.
 __device__ __forceinline__ void phi_two(double a, double b, double& fa, double& fb) {
     const double c = -2.0402788931935790;  // -sqrt2 log2(e)
     const double da = 1.0 + exp2_neg(c * fabs(a)), db = 1.0 + exp2_neg(c * fabs(b));
@@ -127,8 +127,8 @@ constexpr int OBS_QUEUE = 64 + 4 * 32;
 // what a thread, a warp and a block sum before the terms are formed
 template <typename T> struct ObsSums {
     long long liq, sol, near, bad;          // cells
-    T l_hi, l_lo, s_hi, s_lo, n_hi, n_lo;   // U over the liquid, the solid, near the interface
-    double phi, phiu;                       // phi and phi U near the interface
+    T l_hi, l_lo, s_hi, s_lo;               // U over the liquid, the solid
+    double u, phi, phiu;                    // U, phi and phi U near the interface
     float c, cu;                            // sign - phi and (sign - phi) U in the bulk
 };
 template <typename T> struct ObsShared {
@@ -144,11 +144,12 @@ template <typename T> struct ObsShared {
 // with c = 2 e^{-sqrt2 |psi|} < 2e-11 (the next term is c^2 / 2): with phi = +-1 those
 // cells contribute 1 + (1-k) U (liquid) or k (1 + (1-k) U) (solid) to the solute
 // sum and 0 or 1 to the solid sum; they are counted and their U summed, exactly in
-// FP32 pairs (Knuth's two-sum: hi + lo carries ~48 bits, more than the FP64 sum of
-// these FP32 values keeps), and the sums of c and c U, in FP32, are 1e-16 of a
-// term per cell accurate (c is below FP64 precision from |psi| = 32 on).  The other cells go to a queue of the warp and are evaluated 64 at a
+// FP32 pairs (Knuth's two-sum: hi + lo carries ~48 bits), and the sums of c and c U, in
+// FP32, are 1e-16 of a term per cell accurate (c is below FP64 precision from |psi| =
+// 32 on); FP64 fields take plain FP64 sums.  The other cells, and those with |U| >
+// 1e18, whose sums could leave the FP32 range, go to a queue of the warp and are evaluated 64 at a
 // time, two to a lane, so that no lane idles where the interface crosses a row;
-// each adds phi and phi U to two FP64 sums.  (Five 1024^2 members with
+// each adds U, phi and phi U to three FP64 sums.  (Five 1024^2 members with
 // mature dendrites: 150 us with the library tanh and both FP64 terms in place, 96
 // with the queue and phi_two, 83 with the bulk from 18 instead of 32, 72 with the
 // terms formed once a block instead of once a thread.)  Rows are walked whole (one block per row, threads
@@ -180,15 +181,19 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
     auto evaluate = [&](int n) {
         __syncwarp();
         const bool v0 = lane < n, v1 = lane + 32 < n;
-        const T p0 = v0 ? sh.psi[warp][lane] : T(0), p1 = v1 ? sh.psi[warp][lane + 32] : T(0);
+        // (phi = +-1 to FP64 precision well below |psi| = 40)
+        auto clamp = [](T x) -> T { return fabs(x) > T(40) ? copysign(T(40), x) : x; };
+        const T p0 = v0 ? clamp(sh.psi[warp][lane]) : T(0), p1 = v1 ? clamp(sh.psi[warp][lane + 32]) : T(0);
         const T u0 = v0 ? sh.U[warp][lane] : T(0), u1 = v1 ? sh.U[warp][lane + 32] : T(0);
         double f0, f1;
         phi_two((double)p0, (double)p1, f0, f1);
         if (v0) {
+            z.u += (double)u0;
             z.phi += f0;
             z.phiu = fma(f0, (double)u0, z.phiu);
         }
         if (v1) {
+            z.u += (double)u1;
             z.phi += f1;
             z.phiu = fma(f1, (double)u1, z.phiu);
         }
@@ -201,7 +206,7 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
             z.bad += 1;
             return false;
         }
-        if (fabs(pst) >= T(18)) {
+        if (fabs(pst) >= T(18) && fabs(ut) <= T(1e18)) {
             float c = 0.0f;
             if (fabs(pst) < T(32)) c = copysignf(2.0f * exp2f(-2.0402788931935790f * fabsf((float)pst)), (float)pst);
             z.c += c;
@@ -216,7 +221,6 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
             return false;
         }
         z.near += 1;
-        acc2(z.n_hi, z.n_lo, ut);
         return true;
     };
     // the tip candidate of one cell
@@ -336,8 +340,8 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
         if (liq) pair(z.l_hi, z.l_lo);
         if (sol) pair(z.s_hi, z.s_lo);
         if (near) {
-            pair(z.n_hi, z.n_lo);
             for (int off = from; off > 0; off >>= 1) {
+                z.u += __shfl_down_sync(all, z.u, off);
                 z.phi += __shfl_down_sync(all, z.phi, off);
                 z.phiu += __shfl_down_sync(all, z.phiu, off);
             }
@@ -362,12 +366,11 @@ __device__ void observe_block(const ObsArgs& a, ObsPartial* __restrict__ partial
     tree(W / 2);
     reduce_tip(acc);
     if (lane == 0) {
-        const double u_liq = (double)z.l_hi + (double)z.l_lo, u_sol = (double)z.s_hi + (double)z.s_lo,
-                     u_near = (double)z.n_hi + (double)z.n_lo;
+        const double u_liq = (double)z.l_hi + (double)z.l_lo, u_sol = (double)z.s_hi + (double)z.s_lo;
         // near the interface: sum (1 + k - (1-k) phi) (1 + (1-k) U) / 2 and sum (1 + phi) / 2
         acc.nonfinite = z.bad;
         acc.solute = ((double)z.liq + omk * u_liq) + k * ((double)z.sol + omk * u_sol) +
-                     0.5 * ((1.0 + k) * ((double)z.near + omk * u_near) - omk * (z.phi + omk * z.phiu)) +
+                     0.5 * ((1.0 + k) * ((double)z.near + omk * z.u) - omk * (z.phi + omk * z.phiu)) +
                      0.5 * omk * ((double)z.c + omk * (double)z.cu);
         acc.solid = (double)z.sol + 0.5 * ((double)z.near + z.phi) - 0.5 * (double)z.c;
         partials[blk] = acc;
