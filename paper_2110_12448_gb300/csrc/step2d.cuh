@@ -11,7 +11,10 @@ namespace pf {
 // successor may take free slots at once where there is at most a block per SM;
 // larger grids leave that to their blocks' exit, because blocks that wait in the
 // free slots of a half-full GPU are spread unevenly (1024^2: 14.4 us a step before,
-// 12.7 so, 15.5 with a successor that waits beside it).
+// 12.7 so, 15.5 with a successor that waits beside it).  Fields and grain maps are
+// read by plain loads: non-coherent ones (__ldg) are for memory that nothing
+// writes while the kernel is there, and this one may be there while the kernel ahead
+// still writes (no difference in time: 0-1.4 % on the step workloads).
 constexpr int EARLY_GRID = 152;  // the SMs of GB300
 __device__ __forceinline__ void after_previous() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -195,24 +198,24 @@ template <typename T>
 __device__ __forceinline__ void load_pair(const T* __restrict__ row, int c, int nx, bool vec, bool per, T& a, T& b) {
     c = wrap_once(c, nx, per);
     if (vec && c >= 0 && c + 1 < nx) {
-        const typename Vec2<T>::t v = __ldg(reinterpret_cast<const typename Vec2<T>::t*>(row + PF_CHK(c, nx - 1)));
+        const typename Vec2<T>::t v = *reinterpret_cast<const typename Vec2<T>::t*>(row + PF_CHK(c, nx - 1));
         a = v.x;
         b = v.y;
     } else {
-        a = __ldg(row + PF_CHK(col_idx(c, nx, per), nx));
-        b = __ldg(row + PF_CHK(col_idx(c + 1, nx, per), nx));
+        a = row[PF_CHK(col_idx(c, nx, per), nx)];
+        b = row[PF_CHK(col_idx(c + 1, nx, per), nx)];
     }
 }
 __device__ __forceinline__ void load_grain_pair(const int16_t* __restrict__ row, int c, int nx, bool vec, bool per,
                                                 int& a, int& b) {
     c = wrap_once(c, nx, per);
     if (vec && c >= 0 && c + 1 < nx) {
-        const int v = __ldg(reinterpret_cast<const int*>(row + PF_CHK(c, nx - 1)));
+        const int v = *reinterpret_cast<const int*>(row + PF_CHK(c, nx - 1));
         a = (int)(int16_t)(v & 0xffff);
         b = (int)(int16_t)((unsigned)v >> 16);
     } else {
-        a = __ldg(row + PF_CHK(col_idx(c, nx, per), nx));
-        b = __ldg(row + PF_CHK(col_idx(c + 1, nx, per), nx));
+        a = row[PF_CHK(col_idx(c, nx, per), nx)];
+        b = row[PF_CHK(col_idx(c + 1, nx, per), nx)];
     }
 }
 template <typename T>

@@ -276,7 +276,7 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
 #else
             const float* __restrict__ at = reinterpret_cast<const float*>(reinterpret_cast<const char*>(row + (x0 - 2)) + lo8);
 #endif
-            const float2 v = __ldg(reinterpret_cast<const float2*>(at));
+            const float2 v = *reinterpret_cast<const float2*>(at);
             return mk(v.x, v.y);
         }
         float a, b;

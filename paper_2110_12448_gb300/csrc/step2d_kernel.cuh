@@ -280,12 +280,12 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
             const T* __restrict__ at = reinterpret_cast<const T*>(reinterpret_cast<const char*>(row + (x0 - 2)) + lo);
 #endif
             if constexpr (ACC == PAIRS) {
-                const typename Vec2<T>::t v = __ldg(reinterpret_cast<const typename Vec2<T>::t*>(at));
+                const typename Vec2<T>::t v = *reinterpret_cast<const typename Vec2<T>::t*>(at);
                 a = v.x;
                 b = v.y;
             } else {
-                a = __ldg(at);
-                b = __ldg(at + 1);
+                a = at[0];
+                b = at[1];
             }
         } else {
             load_pair<T>(row, cL, nx, vec, per, a, b);
@@ -384,7 +384,7 @@ __device__ __forceinline__ void sweep2d(const WorkItem& wi, const InstRec& rec, 
     auto fetch_grain = [&](int row) -> int {
         if constexpr (FR == FR_ONE) return 0;
         const int16_t* __restrict__ at = grain + (size_t)PF_CHK(row, ny) * nx;
-        if constexpr (ACC == PAIRS) return __ldg(reinterpret_cast<const int*>(at + PF_CHK(cL, nx - 1)));
+        if constexpr (ACC == PAIRS) return *reinterpret_cast<const int*>(at + PF_CHK(cL, nx - 1));
         int a, b;
         load_grain_pair(at, cL, nx, vec, per, a, b);
         return (a & 0xffff) | (b << 16);

@@ -156,10 +156,10 @@ template <bool PAIRS> struct Where {
     }
     template <typename T> __device__ __forceinline__ V<T> load(const T* __restrict__ plane, long long o) const {
         if constexpr (PAIRS) {
-            const typename Vec2<T>::t v = __ldg(reinterpret_cast<const typename Vec2<T>::t*>(plane + o));
+            const typename Vec2<T>::t v = *reinterpret_cast<const typename Vec2<T>::t*>(plane + o);
             return mk(v.x, v.y);
         }
-        return mk(__ldg(plane + o), __ldg(plane + o + db));
+        return mk(plane[o], plane[o + db]);
     }
     template <typename T> __device__ __forceinline__ void store(T* __restrict__ plane, V<T> v) const {
         if (PAIRS && okL && okR) {
