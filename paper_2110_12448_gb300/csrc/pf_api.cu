@@ -1150,54 +1150,61 @@ int group_rebuild(pf_group* g) {
         recs.push_back(make_rec(s, (int)((s->step ^ g->launches) & 1)));
         g->gens.push_back(s->rec_gen);
     }
-    // Sweeps: a member's own, but the 2D members of a class whose tiles nobody
-    // has set share one that suits the whole launch (a cell's bits do not depend
-    // on it); in a wavefront's bands, one of at least 8 rows.
+    // depth 2 applies when no member has a frozen temperature or the two-kernel form
+    g->wave = g->depth == 2;
+    for (const pf_sim* s : g->members)
+        if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.kernels == PF_TWO_KERNELS) g->wave = false;
+    // Sweeps (a cell's bits do not depend on them): a member's own where its tile
+    // was set.  The other 2D members of a class share one that suits the whole launch,
+    // out of what the members' own choices take of the work list and what all of them
+    // leave of it, 32 rows in a wavefront; the other 3D members keep their own.
     std::vector<int> sweep(g->members.size());
-    for (size_t m = 0; m < g->members.size(); ++m) sweep[m] = g->members[m]->sweep;
-    auto shares = [&](int i) {
-        const pf_sim* s = g->members[i];
-        return s->auto_tile && s->p.dim == 2;
+    auto items_of = [&](size_t m, int sw) -> long long {
+        const pf_sim* s = g->members[m];
+        const Strips v = strips_of(&s->p, s->bx, s->by);
+        return (long long)v.columns * cdiv(v.extent, sw);
     };
-    for (size_t a = 0; a < order.size();) {
+    auto items = [&]() {
+        long long n = 0;
+        for (size_t m = 0; m < g->members.size(); ++m) n += items_of(m, sweep[m]);
+        return n;
+    };
+    for (size_t m = 0; m < g->members.size(); ++m)
+        sweep[m] = g->wave && g->members[m]->auto_tile && g->members[m]->p.dim == 2 ? 32 : g->members[m]->sweep;
+    for (size_t a = 0; a < order.size() && !g->wave;) {
         size_t b = a;
         std::vector<Strips> v;
-        for (; b < order.size() && key(order[b]) == key(order[a]); ++b)
-            if (shares(order[b])) v.push_back(strips_of(&g->members[order[b]]->p, 64, 1));
+        std::vector<int> sharers;
+        for (; b < order.size() && key(order[b]) == key(order[a]); ++b) {
+            const pf_sim* s = g->members[order[b]];
+            if (!s->auto_tile || s->p.dim != 2) continue;
+            v.push_back(strips_of(&s->p, s->bx, s->by));
+            sharers.push_back(order[b]);
+        }
         if (!v.empty()) {
             // other groups' launches usually fill the tail (batch.Batch)
             SweepModel model = sweep_model(&g->members[order[a]]->p);
             if (v.size() > 1) model.tail = 0.2;
-            const int s = g->depth == 2 ? 32 : pick_sweep(model, v, g->max_work);
-            for (; a < b; ++a)
-                if (s > 0 && shares(order[a])) sweep[order[a]] = s;
+            long long budget = std::max(0LL, g->max_work - items());
+            for (int m : sharers) budget += items_of(m, sweep[m]);
+            budget = std::min(budget, (long long)g->max_work);
+            const int pick = pick_sweep(model, v, budget);
+            if (pick > 0)
+                for (int m : sharers) sweep[m] = pick;
         }
         a = b;
     }
-    // A work list sized for longer sweeps than the defaults: the 3D members whose
-    // tiles nobody has set sweep further (their bits may depend on it).
-    auto items = [&]() {
-        long long n = 0;
+    // A work list sized for longer sweeps: the members whose tiles nobody has set
+    // sweep further, in 2D up to a little beyond the longest default.
+    for (int longer = 32; items() > g->max_work && longer <= 1 << 14; longer += std::max(1, longer / 16))
         for (size_t m = 0; m < g->members.size(); ++m) {
             const pf_sim* s = g->members[m];
-            const Strips v = strips_of(&s->p, s->bx, s->by);
-            n += (long long)v.columns * cdiv(v.extent, sweep[m]);
+            if (s->auto_tile && (s->p.dim == 3 || longer <= 64)) sweep[m] = std::max(sweep[m], longer);
         }
-        return n;
-    };
-    for (int longer = 32; items() > g->max_work && longer <= 1 << 14; longer *= 2)
-        for (size_t m = 0; m < g->members.size(); ++m)
-            if (g->members[m]->auto_tile && g->members[m]->p.dim == 3) sweep[m] = std::max(sweep[m], longer);
+    // a band must be at least two rows high (the 2D psi halo; 3D planes: one)
+    for (size_t m = 0; m < g->members.size(); ++m)
+        if ((long long)g->band_sweeps * sweep[m] < 2) g->wave = false;
     long long prev = -1;
-    // depth 2 applies when no member has a frozen temperature or the
-    // two-kernel form; a band must be at least two rows high (the psi halo),
-    // which sweeps of at least 8 rows already guarantee
-    g->wave = g->depth == 2;
-    for (size_t m = 0; m < g->members.size(); ++m) {
-        const pf_sim* s = g->members[m];
-        if (s->p.thermal == PF_FROZEN_GRADIENT || s->p.kernels == PF_TWO_KERNELS || (long long)g->band_sweeps * sweep[m] < 2)
-            g->wave = false;
-    }
     g->n_bands = 0;
     std::vector<int> band_of;  // depth 2: band of every work item, in work order
     for (int i : order) {
