@@ -287,10 +287,12 @@ int pf_device_fields(pf_sim* s, void** psi, void** U, void** grain);
 
 /* Tile shape of the step: the widths along x and y (2D: 64 x 1 columns of a
  * warp; 3D: a block shape of the documented list) and the number of rows (2D)
- * or planes (3D) one work item sweeps; 0 keeps the current value.  Until a
- * sweep is set here the library chooses it from the grid (and, in a group,
- * from all members), and pf_get_tile reports its choice.  In 2D
- * the results do not depend on the sweep.  Used by the autotuner. */
+ * or planes (3D) one work item sweeps, at least 2 rows or 4 planes; 0 keeps the
+ * current value.  Until a sweep is set here the library chooses it from the grid
+ * and the block shape (in a group from the members of a class, and for what the
+ * group's work list holds), and pf_get_tile reports its choice for the instance
+ * alone; a tile reported for one handle can be set on any other of its
+ * dimension.  The results do not depend on the sweep.  Used by the autotuner. */
 int pf_set_tile(pf_sim* s, int block_x, int block_y, int sweep);
 int pf_get_tile(pf_sim* s, int* block_x, int* block_y, int* sweep);
 /* Work units of the current tile that are resident on the device at once

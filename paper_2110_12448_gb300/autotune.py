@@ -10,7 +10,9 @@ work per work item), so the answer depends on the batch size as well as the
 grid.  Besides a fixed list, the candidates include, for k = 1, 2, ... waves,
 the shortest sweep whose work list fits in k waves of resident units
 (``pf_resident_units``), which balances the persistent launch with the least
-prologue for that wave count.
+prologue for that wave count.  All are of at least 8 rows: grids that leave the
+GPU partly empty run faster at the library's own choice, which is shorter there
+(down to 2 rows or 4 planes), and need no tuning.
 
 It also races the temporal-blocking depth (``pf_group_set_depth``): depth 2
 advances two steps per wavefront over bands of sweeps, so that the

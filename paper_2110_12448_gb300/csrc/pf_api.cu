@@ -160,17 +160,23 @@ int pick_sweep(const SweepModel& m, const std::vector<Strips>& v, long long max_
 struct Tile {
     int bx, by, sweep;
 };
+int default_sweep(const pf_params* p, int bx, int by) {
+    return pick_sweep(sweep_model(p), {strips_of(p, bx, by)}, LLONG_MAX);
+}
 Tile default_tile(const pf_params* p) {
-    Tile t = p->dim == 2 ? Tile{64, 1, 32}    // one warp per 60-column strip
-                         : Tile{34, 10, 32};  // (TX + 4, TY + 4): 30 x 6 output columns
-    t.sweep = pick_sweep(sweep_model(p), {strips_of(p, t.bx, t.by)}, LLONG_MAX);
+    Tile t = p->dim == 2 ? Tile{64, 1, 0}    // one warp per 60-column strip
+                         : Tile{34, 10, 0};  // (TX + 4, TY + 4): 30 x 6 output columns
+    t.sweep = default_sweep(p, t.bx, t.by);
     return t;
 }
+// the shortest sweep that pf_set_tile takes: the shortest the library chooses for any grid
+int min_sweep(const pf_params* p) { return sweep_model(p).lo; }
 
-// capacity of the work list: the smallest tile that pf_set_tile takes, or the default
+// capacity of the work list: sweeps of min_sweep on the narrowest block, so that any
+// handle takes the tile of any other
 int max_work_items(const pf_params* p) {
-    if (p->dim == 3) return cdiv(p->nx, 12) * cdiv(p->ny, 4) * cdiv(p->nz, 4);
-    return std::max(cdiv(p->nx, 60) * cdiv(p->ny, 8), cdiv(p->nx, 60) * cdiv(p->ny, default_tile(p).sweep));
+    if (p->dim == 3) return cdiv(p->nx, 12) * cdiv(p->ny, 4) * cdiv(p->nz, min_sweep(p));
+    return cdiv(p->nx, 60) * cdiv(p->ny, min_sweep(p));
 }
 
 // whether d psi/dt travels between the passes in device memory: the 2D two-kernel
@@ -934,8 +940,9 @@ int pf_set_tile(pf_sim* s, int block_x, int block_y, int sweep) {
     if (block_x) s->bx = block_x;
     if (block_y) s->by = block_y;
     if (sweep) s->sweep = sweep;
-    bool ok = (sweep == 0 || (sweep >= 8 && sweep <= 1 << 20)) && occupancy(s) > 0;
+    bool ok = (sweep == 0 || (sweep >= min_sweep(&s->p) && sweep <= 1 << 20)) && occupancy(s) > 0;
     if (ok) {
+        if (sweep == 0 && s->auto_tile) s->sweep = default_sweep(&s->p, s->bx, s->by);
         std::vector<WorkItem> tmp;
         build_work(s, 0, s->sweep, tmp);
         ok = (int)tmp.size() <= s->L.max_work;
