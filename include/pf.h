@@ -382,15 +382,15 @@ int pf_group_size(const pf_group* g);
  * only level n).  depth 1 (the default) launches every step over whole grids.
  * depth 2 advances two steps per wavefront over bands along the sweep axis
  * (2D: y, 3D: z), band_sweeps work-item sweeps high (per member:
- * band_sweeps x its sweep rows):
+ * band_sweeps x its sweep rows, 32 where no sweep was set):
  *   step n+1 on band 0, step n+1 on band 1, step n+2 on band 0,
  *   step n+1 on band 2, step n+2 on band 1, ..., step n+2 on the last band
  * (pf_wavefront_order), all on the group's stream.  Step n+2 on band b reads
  * level n+1 on band b and two rows (planes) into its neighbours, which the
  * step n+1 launches before it have written and no later launch overwrites; it
  * writes level n+2 only into band b, which no later step n+1 launch reads,
- * since a band (at least one sweep of at least 8 rows) is higher than the
- * two-row psi halo.  The intermediate level is then read back while it is
+ * since a band is at least as high as the two-row psi halo (sweeps are at least
+ * 2 rows; 3D: 4 planes, for reads one plane into each neighbour).  The intermediate level is then read back while it is
  * still in L2.  Every cell gets the same arithmetic as at depth 1, so results
  * are bit-identical.  A group whose members include a frozen temperature (one
  * step clock per launch) or a two-kernel member (its U pass needs the psi

@@ -1164,7 +1164,8 @@ int group_rebuild(pf_group* g) {
     // Sweeps (a cell's bits do not depend on them): a member's own where its tile
     // was set.  The other 2D members of a class share one that suits the whole launch,
     // out of what the members' own choices take of the work list and what all of them
-    // leave of it, 32 rows in a wavefront; the other 3D members keep their own.
+    // leave of it; the other 3D members keep their own.  In a wavefront every sweep of
+    // a band is part of a launch of its own: 32 rows or planes.
     std::vector<int> sweep(g->members.size());
     auto items_of = [&](size_t m, int sw) -> long long {
         const pf_sim* s = g->members[m];
@@ -1177,7 +1178,7 @@ int group_rebuild(pf_group* g) {
         return n;
     };
     for (size_t m = 0; m < g->members.size(); ++m)
-        sweep[m] = g->wave && g->members[m]->auto_tile && g->members[m]->p.dim == 2 ? 32 : g->members[m]->sweep;
+        sweep[m] = g->wave && g->members[m]->auto_tile ? 32 : g->members[m]->sweep;
     for (size_t a = 0; a < order.size() && !g->wave;) {
         size_t b = a;
         std::vector<Strips> v;
