@@ -139,7 +139,9 @@ typedef struct {
 } pf_seed;
 
 /* Observation (tip tracking of Sec. 3.3.2 and 6.2.2, solute integral of
- * Eq. Supersaturation).  All reductions run in FP64 on the device. */
+ * Eq. Supersaturation).  Reductions run in FP64 on the device; the terms of cells
+ * of FP32 fields far from the interface (|psi| >= 18, |U| <= 1e18) are first summed
+ * in FP32 pairs of about 48 bits. */
 typedef struct {
     int64_t step;             /* steps taken by the handle */
     double t;                 /* step * dt */

@@ -119,7 +119,7 @@ int kprec(const pf_params& p) { return p.precision == PF_F64 ? 1 : (p.precision 
 // 24.7 against 6.2, 1024^2 24.7 / 16.5, 200^2 FP64 529 / 72, 600 x 500 FP64 529 /
 // 192, 64^3 61 / 24, 96^3 74 / 43, 128^3 87 / 68; where the GPU is full anyway the
 // choice costs little (2048^2 39.0 / 39.0, 256^3 379 / 384).
-// (Since then launches overlap, step2d.cuh: 128^2 4.6, 1024^2 12.7, 200^2 FP64 69.)
+// (Since then launches overlap, step2d.cuh: 128^2 4.6, 1024^2 12.8, 200^2 FP64 70.)
 struct SweepModel {
     int units, resident, lo, hi, by;  // resident: items a unit; lo, hi, by: the sweep lengths tried
     double ov, fill, tail;
@@ -348,8 +348,6 @@ InstRec make_rec(const pf_sim* s, int parity_offset) {
     c[C_HH] = h * h;
     c[C_IH2] = 1.0 / (h * h);
     c[C_I6H2] = 1.0 / (6.0 * h * h);
-    c[C_G10] = 2.0 / 3.0 / (4.0 * h * h);
-    c[C_G01] = 1.0 / 3.0 / (8.0 * h * h);
     c[C_DT] = s->p.dt;
     c[C_K] = s->p.k;
     c[C_OMK] = 1.0 - s->p.k;
@@ -357,7 +355,6 @@ InstRec make_rec(const pf_sim* s, int parity_offset) {
     c[C_LAM] = s->p.lambda;
     c[C_D] = s->p.D;
     c[C_ISQ2DT] = 1.0 / (1.41421356237309504880 * s->p.dt);
-    c[C_I4H2] = 1.0 / (4.0 * h * h);
     c[C_OPK] = 1.0 + s->p.k;
     const double sq2 = 1.41421356237309504880;
     c[C_DTL21] = s->p.dt / (6.0 * h * h);

@@ -18,8 +18,6 @@ enum : int {
     C_HH,        // h^2
     C_IH2,       // 1/h^2
     C_I6H2,      // 1/(6h^2)
-    C_G10,       // (2/3)/(4h^2)
-    C_G01,       // (1/3)/(8h^2)
     C_DT,        // dt
     C_K,         // k
     C_OMK,       // 1-k
@@ -27,7 +25,6 @@ enum : int {
     C_LAM,       // lambda
     C_D,         // D
     C_ISQ2DT,    // 1/(sqrt2 dt)
-    C_I4H2,      // 1/(4h^2)
     C_OPK,       // 1+k
     C_DTL21,     // dt / (6h^2): Eq. PF_a in units of 1/(6h^2)
     C_DTL10,     // dt / h^2
@@ -60,7 +57,7 @@ struct InstRec {
     int32_t bcx;      // 1: periodic x (2D)
     int32_t tlevel;   // 1: T0 time level (pure forward Euler of Eq. PF_b)
     int32_t n_grains; // rows of the rotation table
-    int32_t one_grain; // 1: every cell is in grain 0 (the grain map need not be read)
+    int32_t one_grain; // 1: every cell is in grain 0 (the compensated kernel then reads no grain map)
     int32_t pad_;
     double h, dt, k, eps4, lambda, D;
     // frozen temperature: zeta(row j, step n) = j zA - zB - n zC

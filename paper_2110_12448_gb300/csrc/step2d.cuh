@@ -11,7 +11,7 @@ namespace pf {
 // successor may take free slots at once where there is at most a block per SM;
 // larger grids leave that to their blocks' exit, because blocks that wait in the
 // free slots of a half-full GPU are spread unevenly (1024^2: 14.4 us a step before,
-// 12.7 so, 15.5 with a successor that waits beside it).  Fields and grain maps are
+// 12.8 so, 15.5 with a successor that waits beside it).  Fields and grain maps are
 // read by plain loads: non-coherent ones (__ldg) are for memory that nothing
 // writes while the kernel is there, and this one may be there while the kernel ahead
 // still writes (no difference in time: 0-1.4 % on the step workloads).
@@ -21,7 +21,7 @@ __device__ __forceinline__ void after_previous() {
     if (gridDim.x <= EARLY_GRID) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 // Launches a step kernel so (programmatic stream serialisation; a capture keeps
-// it as an edge of the graph).  128^2: 6.2 -> 4.6 us a step; 200^2 FP64 72 -> 69;
+// it as an edge of the graph).  128^2: 6.2 -> 4.6 us a step; 200^2 FP64 72 -> 70;
 // full grids gain under 1 %.
 template <typename... P, typename... A>
 void launch_next(void (*k)(P...), int grid, int threads, size_t smem, cudaStream_t st, A... args) {
@@ -149,6 +149,12 @@ __device__ __forceinline__ V<double> fma(V<double> a, V<double> b, V<double> c) 
 }
 template <typename T> __device__ __forceinline__ V<T> rcp2(V<T> a) { return mk(M<T>::rcp(a.x()), M<T>::rcp(a.y())); }
 
+// f of each column
+template <typename T, typename F> __device__ __forceinline__ V<T> each(V<T> a, F f) { return mk(f(a.x()), f(a.y())); }
+template <typename T, typename F> __device__ __forceinline__ V<T> each(V<T> a, V<T> b, F f) {
+    return mk(f(a.x(), b.x()), f(a.y(), b.y()));
+}
+
 template <typename T> __device__ __forceinline__ T shup(T v) { return __shfl_up_sync(FULL, v, 1); }
 template <typename T> __device__ __forceinline__ T shdn(T v) { return __shfl_down_sync(FULL, v, 1); }
 
@@ -229,6 +235,42 @@ __device__ __forceinline__ void store_pair(T* __restrict__ row, int c, int nx, b
         if (okL) row[PF_CHK(c, nx)] = v.x();
         if (okR) row[PF_CHK(c + 1, nx)] = v.y();
     }
+}
+
+// App. B: |grad b| at a <10> face (pairs); B(p, q) = b at origin + p normal + q tangent.
+template <typename T, typename F> __device__ __forceinline__ V<T> appb_face2(F B, T ih) {
+    const V<T> a1 = B(1, 1) - B(0, -1), a2 = B(0, 1) - B(1, -1);
+    const V<T> b1 = B(2, 1) - B(-1, -1), b2 = B(-1, 1) - B(2, -1);
+    const V<T> c1 = B(1, 2) - B(0, -2), c2 = B(0, 2) - B(1, -2);
+    const V<T> dn = (bc<T>(T(35.0 / 48.0)) * (a1 - a2) - bc<T>(T(1.0 / 48.0)) * (b1 - b2) -
+                     bc<T>(T(1.0 / 6.0)) * (c1 - c2)) * bc<T>(ih);
+    const V<T> dt = (bc<T>(T(35.0 / 96.0)) * (a1 + a2) - bc<T>(T(1.0 / 32.0)) * (b1 + b2) -
+                     bc<T>(T(1.0 / 24.0)) * (c1 + c2)) * bc<T>(ih);
+    const V<T> m2 = fma(dn, dn, dt * dt);
+    return each(m2, [](T m) { return M<T>::sqrt_(m); });
+}
+// App. B: |grad b| at a corner; B(p, q) = b at origin + p x + q y.
+template <typename T, typename F> __device__ __forceinline__ V<T> appb_corner2(F B, T ih) {
+    const V<T> a1 = B(1, 1) - B(0, 0), a2 = B(0, 1) - B(1, 0);
+    const V<T> b1 = B(2, 1) - B(-1, 0), b2 = B(-1, 1) - B(2, 0);
+    const V<T> c1 = B(1, 2) - B(0, -1), c2 = B(0, 2) - B(1, -1);
+    const V<T> dx = (bc<T>(T(5.0 / 8.0)) * (a1 - a2) - bc<T>(T(1.0 / 48.0)) * (b1 - b2) -
+                     bc<T>(T(1.0 / 16.0)) * (c1 - c2)) * bc<T>(ih);
+    const V<T> dy = (bc<T>(T(5.0 / 8.0)) * (a1 + a2) - bc<T>(T(1.0 / 16.0)) * (b1 + b2) -
+                     bc<T>(T(1.0 / 48.0)) * (c1 + c2)) * bc<T>(ih);
+    const V<T> m2 = fma(dx, dx, dy * dy);
+    return each(m2, [](T m) { return M<T>::sqrt_(m); });
+}
+// App. B magnitude m at a flux point raised to at least half of the two-point
+// slope |d| s (s = 1 / |e|): the quotient slope / m, the unit normal's
+// component along e, then stays within [-2, 2]; it leaves that range only
+// where grad psi has no direction (reading R-A21G)
+template <typename T> __device__ __forceinline__ V<T> appb_floor2(V<T> m, V<T> d, T s) {
+    return each(m, d, [&](T a, T b) { return fmax(a, T(0.5) * s * fabs(b)); });
+}
+// f / m per column with the guard on |grad psi| of the standard anti-trapping forms
+template <typename T> __device__ __forceinline__ V<T> guarded_div2(V<T> f, V<T> m, T hh) {
+    return each(f * rcp2(m), m, [&](T q, T a) { return a * a * hh < Guard<T>::v ? T(0) : q; });
 }
 
 }  // namespace

@@ -36,7 +36,7 @@ struct Rot2 {
 };
 
 // Normal component of J - g for face gradients (gx, gy) of both columns, J =
-// d(a_s^2 |g|^2 / 2)/dg, without cancellation: crystal components c = R^float g,
+// d(a_s^2 |g|^2 / 2)/dg, without cancellation: crystal components c = R^T g,
 // s_p = c_p^2 / |c|^2, q = s_x^2 + s_y^2, a_s = 1 - 3 eps + 4 eps q; with s_x + s_y = 1 in 2D, a - 1 = eps (4q - 3) =
 // eps (1 - 8 s_x s_y), a^2 - 1 = (a - 1)(a + 1), and s_x - q = s_y (s_x - s_y),
 // s_y - q = -s_x (s_x - s_y), so
@@ -50,13 +50,13 @@ __device__ __forceinline__ V<float> aniso_qn2c(V<float> gx, V<float> gy, const R
     const V<float> inv = rcp2(r2);
     const V<float> sx = cx * cx * inv, sy = cy * cy * inv;
     const V<float> dxy = (cx - cy) * (cx + cy) * inv;  // s_x - s_y
-    const V<float> b = fma(bc<float>(float(-8)) * sx, sy, bc<float>(float(1)));
-    const V<float> a = fma(bc<float>(eps), b, bc<float>(float(1)));
-    const V<float> B = b * fma(bc<float>(eps), b, bc<float>(float(2)));
-    const V<float> t = bc<float>(float(16)) * a * dxy;
-    const V<float> jx = cx * bc<float>(eps) * fma(t, sy, B), jy = cy * bc<float>(eps) * fma(t * bc<float>(float(-1)), sx, B);
+    const V<float> b = fma(bc<float>(-8.0f) * sx, sy, bc<float>(1.0f));
+    const V<float> a = fma(bc<float>(eps), b, bc<float>(1.0f));
+    const V<float> B = b * fma(bc<float>(eps), b, bc<float>(2.0f));
+    const V<float> t = bc<float>(16.0f) * a * dxy;
+    const V<float> jx = cx * bc<float>(eps) * fma(t, sy, B), jy = cy * bc<float>(eps) * fma(t * bc<float>(-1.0f), sx, B);
     const V<float> o = xface ? fma(R.a, jx, R.b * jy) : fma(R.c, jx, R.d * jy);
-    return mk(r2.x() * hh < Guard<float>::v ? float(0) : o.x(), r2.y() * hh < Guard<float>::v ? float(0) : o.y());
+    return mk(r2.x() * hh < Guard<float>::v ? 0.0f : o.x(), r2.y() * hh < Guard<float>::v ? 0.0f : o.y());
 }
 // the anisotropic part 4 eps q of a_s = (1 - 3 eps) + 4 eps q (3 eps where
 // the normal is undefined, so that a_s = 1): the compensated state forms
@@ -67,46 +67,9 @@ __device__ __forceinline__ V<float> aniso_w2(V<float> gx, V<float> gy, const Rot
     const V<float> r2 = fma(cx, cx, cy * cy);
     const V<float> inv = rcp2(r2);
     const V<float> sx = cx * cx * inv, sy = cy * cy * inv;
-    const V<float> w = bc<float>(float(4) * eps) * fma(sx, sx, sy * sy);
-    return mk(r2.x() * hh < Guard<float>::v ? float(3) * eps : w.x(), r2.y() * hh < Guard<float>::v ? float(3) * eps : w.y());
+    const V<float> w = bc<float>(4.0f * eps) * fma(sx, sx, sy * sy);
+    return mk(r2.x() * hh < Guard<float>::v ? 3.0f * eps : w.x(), r2.y() * hh < Guard<float>::v ? 3.0f * eps : w.y());
 }
-// App. B: |grad b| at a <10> face (pairs); B(p, q) = b at origin + p normal + q tangent.
-template <typename F> __device__ __forceinline__ V<float> appb_face2(F B, float ih) {
-    const V<float> a1 = B(1, 1) - B(0, -1), a2 = B(0, 1) - B(1, -1);
-    const V<float> b1 = B(2, 1) - B(-1, -1), b2 = B(-1, 1) - B(2, -1);
-    const V<float> c1 = B(1, 2) - B(0, -2), c2 = B(0, 2) - B(1, -2);
-    const V<float> dn = (bc<float>(float(35.0 / 48.0)) * (a1 - a2) - bc<float>(float(1.0 / 48.0)) * (b1 - b2) -
-                     bc<float>(float(1.0 / 6.0)) * (c1 - c2)) * bc<float>(ih);
-    const V<float> dt = (bc<float>(float(35.0 / 96.0)) * (a1 + a2) - bc<float>(float(1.0 / 32.0)) * (b1 + b2) -
-                     bc<float>(float(1.0 / 24.0)) * (c1 + c2)) * bc<float>(ih);
-    const V<float> m2 = fma(dn, dn, dt * dt);
-    return mk(M<float>::sqrt_(m2.x()), M<float>::sqrt_(m2.y()));
-}
-// App. B: |grad b| at a corner; B(p, q) = b at origin + p x + q y.
-template <typename F> __device__ __forceinline__ V<float> appb_corner2(F B, float ih) {
-    const V<float> a1 = B(1, 1) - B(0, 0), a2 = B(0, 1) - B(1, 0);
-    const V<float> b1 = B(2, 1) - B(-1, 0), b2 = B(-1, 1) - B(2, 0);
-    const V<float> c1 = B(1, 2) - B(0, -1), c2 = B(0, 2) - B(1, -1);
-    const V<float> dx = (bc<float>(float(5.0 / 8.0)) * (a1 - a2) - bc<float>(float(1.0 / 48.0)) * (b1 - b2) -
-                     bc<float>(float(1.0 / 16.0)) * (c1 - c2)) * bc<float>(ih);
-    const V<float> dy = (bc<float>(float(5.0 / 8.0)) * (a1 + a2) - bc<float>(float(1.0 / 16.0)) * (b1 + b2) -
-                     bc<float>(float(1.0 / 48.0)) * (c1 + c2)) * bc<float>(ih);
-    const V<float> m2 = fma(dx, dx, dy * dy);
-    return mk(M<float>::sqrt_(m2.x()), M<float>::sqrt_(m2.y()));
-}
-// App. B magnitude m at a flux point raised to at least half of the two-point
-// slope |d| s (s = 1 / |e|): the quotient slope / m, the unit normal's
-// component along e, then stays within [-2, 2]; it leaves that range only
-// where grad psi has no direction (reading R-A21G)
-__device__ __forceinline__ V<float> appb_floor2(V<float> m, V<float> d, float s) {
-    return mk(fmax(m.x(), float(0.5) * s * fabs(d.x())), fmax(m.y(), float(0.5) * s * fabs(d.y())));
-}
-// f / m per column with the guard on |grad psi| of the standard anti-trapping forms
-__device__ __forceinline__ V<float> guarded_div2(V<float> f, V<float> m, float hh) {
-    const V<float> q = f * rcp2(m);
-    return mk(m.x() * m.x() * hh < Guard<float>::v ? float(0) : q.x(), m.y() * m.y() * hh < Guard<float>::v ? float(0) : q.y());
-}
-
 // (hi, lo) + d: Knuth's two-sum of hi and d, the rounding error folded into
 // lo, renormalised by Dekker's fast two-sum (the _rn intrinsics are never
 // contracted into FMAs, which would break the error-free transformations)
@@ -493,8 +456,8 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
                     const V2 gx = dxp * k_(ih), gy = ((P0.E + P0.C) - (Q.E + Q.C)) * k_(i4h);
                     const V2 yx = ((P0.E + Pm.E) - (P0.W + Pm.W)) * k_(i4h), yy = dyp * k_(ih);
                     const V2 mx = fma(gx, gx, gy * gy), my = fma(yx, yx, yy * yy);
-                    const V2 fxA = guarded_div2(half * (AA0.C + AA0.E) * dxp, mk(M<float>::sqrt_(mx.x()), M<float>::sqrt_(mx.y())), hh);
-                    const V2 fyA = guarded_div2(half * (AA0.C + AA1.C) * dyp, mk(M<float>::sqrt_(my.x()), M<float>::sqrt_(my.y())), hh);
+                    const V2 fxA = guarded_div2<float>(half * (AA0.C + AA0.E) * dxp, mk(M<float>::sqrt_(mx.x()), M<float>::sqrt_(mx.y())), hh);
+                    const V2 fyA = guarded_div2<float>(half * (AA0.C + AA1.C) * dyp, mk(M<float>::sqrt_(my.x()), M<float>::sqrt_(my.y())), hh);
                     sA = (fxA - from_west(fxA)) + (fyA - yA);
                     yA = fyA;
                 } else {
@@ -541,10 +504,10 @@ __device__ __forceinline__ void sweep2c(const WorkItem& wi, const InstRec& rec, 
                         }
                         auto ps = [&](int i, int j) -> V2 { return Q[2 + j].pat(i); };
                         const float ihd = ih * 0.70710678118654752440f;  // 1 / |e| of the <11> fluxes
-                        fx = guarded_div2(fx, appb_floor2(appb_face2([&](int i, int j) { return ps(i, j); }, ih), dx, ih), hh);
-                        fy = guarded_div2(fy, appb_floor2(appb_face2([&](int i, int j) { return ps(j, i); }, ih), dy, ih), hh);
-                        pp = guarded_div2(pp, appb_floor2(appb_corner2([&](int i, int j) { return ps(i, j); }, ih), dpp, ihd), hh);
-                        mp = guarded_div2(mp, appb_floor2(appb_corner2([&](int i, int j) { return ps(i - 1, j); }, ih), dmp, ihd), hh);
+                        fx = guarded_div2<float>(fx, appb_floor2<float>(appb_face2<float>([&](int i, int j) { return ps(i, j); }, ih), dx, ih), hh);
+                        fy = guarded_div2<float>(fy, appb_floor2<float>(appb_face2<float>([&](int i, int j) { return ps(j, i); }, ih), dy, ih), hh);
+                        pp = guarded_div2<float>(pp, appb_floor2<float>(appb_corner2<float>([&](int i, int j) { return ps(i, j); }, ih), dpp, ihd), hh);
+                        mp = guarded_div2<float>(mp, appb_floor2<float>(appb_corner2<float>([&](int i, int j) { return ps(i - 1, j); }, ih), dmp, ihd), hh);
                     }
                     sA = gather(fx, fy, pp, mp, yA, mmA, pmA);
                 } else {

@@ -66,12 +66,6 @@
 namespace pf {
 namespace {
 
-// f of each column
-template <typename T, typename F> __device__ __forceinline__ V<T> each(V<T> a, F f) { return mk(f(a.x()), f(a.y())); }
-template <typename T, typename F> __device__ __forceinline__ V<T> each(V<T> a, V<T> b, F f) {
-    return mk(f(a.x(), b.x()), f(a.y(), b.y()));
-}
-
 // Which crystal frames an instance has: FR_ONE every cell in grain 0, the
 // frame orthonormal (no grain rows are read); FR_CELL per-cell grains,
 // orthonormal frames; FR_ANY any matrices (J - g by rotation into the frame
@@ -156,56 +150,21 @@ __device__ __forceinline__ V<T> aniso_as(V<T> gx, V<T> gy, V<T> inv, const Frame
     }
 }
 
-// App. B: |grad b| at a <10> face (pairs); B(p, q) = b at origin + p normal + q tangent.
-template <typename T, typename F> __device__ __forceinline__ V<T> appb_face2(F B, T ih) {
-    const V<T> a1 = B(1, 1) - B(0, -1), a2 = B(0, 1) - B(1, -1);
-    const V<T> b1 = B(2, 1) - B(-1, -1), b2 = B(-1, 1) - B(2, -1);
-    const V<T> c1 = B(1, 2) - B(0, -2), c2 = B(0, 2) - B(1, -2);
-    const V<T> dn = (bc<T>(T(35.0 / 48.0)) * (a1 - a2) - bc<T>(T(1.0 / 48.0)) * (b1 - b2) -
-                     bc<T>(T(1.0 / 6.0)) * (c1 - c2)) * bc<T>(ih);
-    const V<T> dt = (bc<T>(T(35.0 / 96.0)) * (a1 + a2) - bc<T>(T(1.0 / 32.0)) * (b1 + b2) -
-                     bc<T>(T(1.0 / 24.0)) * (c1 + c2)) * bc<T>(ih);
-    const V<T> m2 = fma(dn, dn, dt * dt);
-    return each(m2, [](T m) { return M<T>::sqrt_(m); });
-}
-// App. B: |grad b| at a corner; B(p, q) = b at origin + p x + q y.
-template <typename T, typename F> __device__ __forceinline__ V<T> appb_corner2(F B, T ih) {
-    const V<T> a1 = B(1, 1) - B(0, 0), a2 = B(0, 1) - B(1, 0);
-    const V<T> b1 = B(2, 1) - B(-1, 0), b2 = B(-1, 1) - B(2, 0);
-    const V<T> c1 = B(1, 2) - B(0, -1), c2 = B(0, 2) - B(1, -1);
-    const V<T> dx = (bc<T>(T(5.0 / 8.0)) * (a1 - a2) - bc<T>(T(1.0 / 48.0)) * (b1 - b2) -
-                     bc<T>(T(1.0 / 16.0)) * (c1 - c2)) * bc<T>(ih);
-    const V<T> dy = (bc<T>(T(5.0 / 8.0)) * (a1 + a2) - bc<T>(T(1.0 / 16.0)) * (b1 + b2) -
-                     bc<T>(T(1.0 / 48.0)) * (c1 + c2)) * bc<T>(ih);
-    const V<T> m2 = fma(dx, dx, dy * dy);
-    return each(m2, [](T m) { return M<T>::sqrt_(m); });
-}
-// App. B magnitude m at a flux point raised to at least half of the two-point
-// slope |d| s (s = 1 / |e|): the quotient slope / m, the unit normal's
-// component along e, then stays within [-2, 2]; it leaves that range only
-// where grad psi has no direction (reading R-A21G)
-template <typename T> __device__ __forceinline__ V<T> appb_floor2(V<T> m, V<T> d, T s) {
-    return each(m, d, [&](T a, T b) { return fmax(a, T(0.5) * s * fabs(b)); });
-}
-// f / m per column with the guard on |grad psi| of the standard anti-trapping forms
-template <typename T> __device__ __forceinline__ V<T> guarded_div2(V<T> f, V<T> m, T hh) {
-    return each(f * rcp2(m), m, [&](T q, T a) { return a * a * hh < Guard<T>::v ? T(0) : q; });
-}
-
 // Resident one-warp blocks per SM that the launch bounds of the FP32 kernels
 // ask for: 17 (120 registers) where one crystal frame and no App. B magnitudes
 // are held, else 16 (128).  The row loop advances two rows per pass with one
 // crystal frame, so that the row state moves between registers every other row
 // only; one with per-cell frames, whose two copies outgrow the registers or the
 // instruction cache.  us a step, 10 x 1024^2, sweeps of 32 / 38 rows:
-//   S-bar_21  17 blocks 60.7 / 62.0, 16: 67.6 / 66.0, 18: 61.7 / 63.1
-//   S_10      17 blocks 56.7 / 57.9, 16: 64.0 / 62.5
-//   S_21      (10 x 781^2, 24 rows) 16 blocks 51.0, 17: 70.1
+//   S-bar_21  17 blocks 61.0 / 62.4, 16: 67.6 / 66.0, 18: 61.7 / 63.1
+//   S_10      17 blocks 54.0 / 56.0, 16: 64.0 / 62.5
+//   S_21      (10 x 781^2, 24 rows) 16 blocks 51.2, 17: 70.1
 // (17 blocks are five warps of a scheduler: 96 registers a thread, so that 20 are
 // resident.)
-// 16 polycrystals: 130.5 with 16 blocks and single rows, 161 with 17, 157 with two
+// (The forms not taken were measured with non-coherent loads, worth up to 1.4 %.)
+// 16 polycrystals: 130.8 with 16 blocks and single rows, 161 with 17, 157 with two
 // rows.  Earlier forms of the loop: four columns a lane in 8 blocks of 240
-// registers 114 (60.7 here), three or four rows per pass 79 and 72 (68); an L2
+// registers 114 (61.0 here), three or four rows per pass 79 and 72 (68); an L2
 // prefetch of the rows ahead changes nothing.
 template <int S, int FR> constexpr int BLOCKS_F32 = FR == FR_ONE && S != S21 ? 17 : 16;
 

@@ -10,7 +10,8 @@
 // while one pass has to evaluate the psi rate again on a ring around every
 // tile (1.42 times the cells with 30 x 6 columns), to exchange planes through
 // shared memory under three barriers a plane, and to hold both phases' state:
-// it measured 862 us a step on 256^3 where the two passes take 356 (198 + 160).
+// it measured 862 us a step on 256^3 where the two passes take 364 (356 before the
+// vote on a plane's phase looked for NaN and the fields were read by plain loads).
 //
 // Both passes share one layout.  A warp owns two rows (y, y + 1) of a strip of
 // 32 columns, 16 lanes with a packed pair of columns each, and marches along
