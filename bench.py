@@ -57,6 +57,12 @@ def bytes_per_cell(ws, precision, two=False) -> float:
     return (B_STATE_TWO if two else B_STATE)[precision] + B_GRAIN * graincells / cells
 
 
+def l2_text(cells, precision):
+    """The state that a step reads and writes, and whether it exceeds the L2."""
+    mb = cells * 2 * (4 if precision == "f32" else 8) / 1e6
+    return f"state {mb:.0f} MB read and {mb:.0f} MB written per step, {'>' if 2 * mb > 129 else '<='} 129 MB L2, no flush"
+
+
 def dist_env():
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
@@ -75,11 +81,11 @@ TRAFFIC = {
     # k_step2d<float, S-bar_21> launches of the two five-instance groups, summed (ncu runs them one
     # after the other, so each group's half of the state partly stays in L2)
     "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d_kernel.cuh", "tile": [64, 1, 32],
-                "sha256": "098f4139e44e03eeb712f0d5416d29ffa2525db1fff24bc448fffad75246b895", "bytes": 97869824},
+                "sha256": "d4ab9e3742f9cbf50ec7fd51fe9ce62c8d43dd184ac2c45bb0e306de0eb9c44e", "bytes": 97060096},
     # one step of the 256^3 free dendrite (tile 34 x 10 x 26): the k_psi3d<float, S-bar_120> launch
     # (217 MB) and the k_u3d launch (266 MB), summed
     "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 26],
-                   "sha256": "e5d268a005ad5a36825bf9869cb714f09eaa41a4183e54e2f889451aeacb5a48", "bytes": 482729728},
+                   "sha256": "6ac1dc7ef0873dcebf7f93e4da8c28d484f4f4768bcbf816bf9338678caf9e12", "bytes": 483016192},
 }
 
 
@@ -94,10 +100,10 @@ TRAFFIC = {
 FLOPS = {
     # the two k_step2d<float, S-bar_21> launches of the orientation sweep (10 x 1024^2, tile 64 x 1 x 32)
     "sweep2d": {"source": "paper_2110_12448_gb300/csrc/step2d_kernel.cuh", "tile": [64, 1, 32],
-                "sha256": "098f4139e44e03eeb712f0d5416d29ffa2525db1fff24bc448fffad75246b895", "flop_per_cell": 200.9},
+                "sha256": "d4ab9e3742f9cbf50ec7fd51fe9ce62c8d43dd184ac2c45bb0e306de0eb9c44e", "flop_per_cell": 200.9},
     # k_psi3d<float, S-bar_120> + k_u3d launches of the 256^3 free dendrite (tile 34 x 10 x 26)
     "dendrite3d": {"source": "paper_2110_12448_gb300/csrc/step3d.cu", "tile": [34, 10, 26],
-                   "sha256": "e5d268a005ad5a36825bf9869cb714f09eaa41a4183e54e2f889451aeacb5a48", "flop_per_cell": 502.4},
+                   "sha256": "6ac1dc7ef0873dcebf7f93e4da8c28d484f4f4768bcbf816bf9338678caf9e12", "flop_per_cell": 502.4},
 }
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
@@ -1001,8 +1007,7 @@ def run_native(args):
                                        f"FP64 observe of every instance every {OBS_EVERY} steps and after the last "
                                        f"timed step ({n_observe} inside the timed region)",
                            "cells_per_gpu": cells,
-                           "l2": f"state {cells * 2 * (4 if args.precision == 'f32' else 8) / 1e6:.0f} MB per step "
-                                 f"> 129 MB L2, no flush"},
+                           "l2": l2_text(cells, args.precision)},
                 "roofline": roof, "roofline_alu": roof_alu, "e2e": e2e, "clocks": clocks.summary(),
                 "latency_ms_per_step": {"p50": statistics.median(per_step),
                                         "p99": per_step[min(len(per_step) - 1, int(0.99 * len(per_step)))],
